@@ -17,17 +17,21 @@ namespace cbct {
 
 // ------------------------------------------------------------- forward A x
 
-// 4 rays per lane hold 80 registers (3 CTAs per SM); fewer fit in 64.
-template <typename T, bool COMP, int R, bool VF>
-__global__ void __launch_bounds__(FWD_THREADS, R >= 4 ? 3 : 4)
+// CTAs per SM by rays per lane: the loads of 4 cells (4 rays) or 8 cells (2
+// rays) in flight, 16 to 32 a warp, are worth more than a third or fourth CTA.
+// A x at 512^3 / 768 x 512 / 180 angles: 4 rays 23.5 ms with 4 cells and 2
+// CTAs, 31.6 ms with 2 cells and 3; 2 rays 26.3 ms with 8 cells and 3 CTAs,
+// 29.6 ms with 4 cells and 4.
+template <typename T, bool COMP, int R, bool VF, bool OFF32>
+__global__ void __launch_bounds__(FWD_THREADS, R >= 4 ? 2 : R == 2 ? 3 : 4)
 forward_kernel(DevGeom g, const T *__restrict__ vol, T *__restrict__ proj, Epilogue epi) {
-    __shared__ double red[FWD_THREADS / 32];
+    __shared__ float4 lists[FWD_COLS * FWD_LIST];
     if (epi.stop && *epi.stop) return;
     auto partial_at = [&]() -> double * {
         const size_t b = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
         return epi.partial ? epi.partial + b * TILE_PARTIALS : nullptr;
     };
-    forward_tile<T, COMP, R, VF>(g, vol, proj, epi, blockIdx.x, blockIdx.y, blockIdx.z, partial_at, red);
+    forward_tile<T, COMP, R, VF, OFF32>(g, vol, proj, epi, blockIdx.x, blockIdx.z, blockIdx.y, partial_at, lists);
 }
 
 template <int R>
@@ -39,7 +43,7 @@ count_kernel(DevGeom g, unsigned long long *count) {
     int c = 0;
     if (iu < g.nu) {
         RayAxis rx, ry, rz[R];
-        load_rays<R>(g, blockIdx.z, iu, blockIdx.y * 32 * R, g.nv, rx, ry, rz);
+        load_rays<R>(g, blockIdx.y, iu, blockIdx.z * 32 * R, g.nv, rx, ry, rz);
         auto fetch = [](int) { return 0.0f; };
         auto seg = [&](int, float len, float) { c += len > 0.0f; };
         trace_columns<R>(g, rx, ry, rz, 0, g.nx, 0, g.ny, 0, g.nz, 0, g.nz, g.nx * g.nz, fetch, seg);
@@ -48,9 +52,14 @@ count_kernel(DevGeom g, unsigned long long *count) {
     if (threadIdx.x == 0) atomicAdd(count, (unsigned long long)s);
 }
 
+// x: detector columns / 8, y: angles, z: row groups.  The row groups come last:
+// a group's rays stay in a slab of the volume (about the group's share of the
+// detector's height), which the angles of the group then find in L2.  With the
+// angles last every angle read the whole volume: at 512^3 / 768 x 512 19.5 GB
+// from HBM in 30 angles, 5.1 TB/s.
 dim3 forward_grid(const DevGeom &g) {
     const int rows = 32 * g.fwd_rows;
-    return dim3((g.nu + FWD_COLS - 1) / FWD_COLS, (g.nv + rows - 1) / rows, g.nangles);
+    return dim3((g.nu + FWD_COLS - 1) / FWD_COLS, g.nangles, (g.nv + rows - 1) / rows);
 }
 
 int forward_num_blocks(const DevGeom &g) {
@@ -58,19 +67,26 @@ int forward_num_blocks(const DevGeom &g) {
     return (int)(gr.x * gr.y * gr.z);
 }
 
+// Largest padded volume whose voxels a 32-bit byte offset reaches (FP32 beyond
+// about 1023^3 voxels is larger).
+constexpr uint64_t OFF32_BYTES = (uint64_t)1 << 32;
+
 template <int R, bool VF>
 static void launch_forward_r(const DevGeom &g, const void *x, void *y, cbct_dtype t, const Epilogue &epi,
                              cudaStream_t s) {
     const dim3 grid = forward_grid(g);
     switch (t) {
     case CBCT_F32:
-        forward_kernel<float, false, R, VF><<<grid, FWD_THREADS, 0, s>>>(g, (const float *)x, (float *)y, epi);
+        if ((uint64_t)zf_len(g) * sizeof(float) <= OFF32_BYTES)
+            forward_kernel<float, false, R, VF, true><<<grid, FWD_THREADS, 0, s>>>(g, (const float *)x, (float *)y, epi);
+        else
+            forward_kernel<float, false, R, VF, false><<<grid, FWD_THREADS, 0, s>>>(g, (const float *)x, (float *)y, epi);
         break;
-    case CBCT_F16:
-        forward_kernel<__half, true, R, VF><<<grid, FWD_THREADS, 0, s>>>(g, (const __half *)x, (__half *)y, epi);
+    case CBCT_F16:                  // at most 2^31 elements (validate_geometry_desc)
+        forward_kernel<__half, true, R, VF, true><<<grid, FWD_THREADS, 0, s>>>(g, (const __half *)x, (__half *)y, epi);
         break;
     case CBCT_BF16:
-        forward_kernel<__nv_bfloat16, true, R, VF><<<grid, FWD_THREADS, 0, s>>>(
+        forward_kernel<__nv_bfloat16, true, R, VF, true><<<grid, FWD_THREADS, 0, s>>>(
             g, (const __nv_bfloat16 *)x, (__nv_bfloat16 *)y, epi);
         break;
     }

@@ -8,8 +8,8 @@
 // xy plane, so all of them cross the x and y voxel planes at the same alpha
 // (the x/y tables depend on (a, iu) only).  A warp therefore takes rays of one
 // detector column: lane l follows rows iv0 + r * 32 + l for r = 0..R-1.  The
-// x/y plane stepping is identical in all lanes and is shared by the warp's
-// 32 R rays; each ray only tracks its own z crossings, which are rare
+// sequence of x/y cells is the same in all lanes and is computed once for the
+// warp's 32 R rays; each ray only tracks its own z crossings, which are rare
 // (|dz/d| <= the cone half-angle).  Volumes are read in a z-fastest layout
 // x[j][i][k] so that the lanes of one row group, which sit at ~17 consecutive
 // k of one voxel column, gather one contiguous run.
@@ -224,171 +224,328 @@ __device__ __forceinline__ void load_rays(const DevGeom &g, int a, int iu, int i
     }
 }
 
+// ------------------------------------------------ x/y cells of a column
+//
+// All rays of one detector column cross the x and y planes at the same alphas,
+// so the sequence of x/y cells a warp walks is the same in its 32 lanes.  The
+// lanes compute it together, CELL_CHUNK = 32 crossings at a time: lane l takes
+// the l-th next x plane and the l-th next y plane, finds how many crossings of
+// the other axis come before each (an estimate from the plane spacing, put
+// right by comparing plane_alpha values), and writes its crossings at their
+// ranks of the merged sequence.  An entry of the list is the alpha at which a
+// cell ends and the linear index of the cell's voxel column.  Stepping the two
+// axes in every lane instead took about 40 of the 95 instructions the warp
+// spent per cell; the list takes 3 per cell.
+constexpr int CELL_CHUNK = 32;
+
+struct CellList {
+    RayAxis rx, ry;
+    float rxn, ryn;          // next plane of each axis, relative to pq
+    float sx, sy;            // +1 / -1, 0 when the column is parallel to the axis' planes
+    float ix, iy;            // planes per alpha (0 when parallel)
+    unsigned col;            // voxel column of the current cell (zf_col)
+    unsigned dcx, dcy;       // its change across an x / y plane
+    unsigned colmax;         // largest column index
+    float amax;
+};
+
+// Sets the list up for the box [0, nx) x [0, ny); false (warp-uniform) if the
+// column misses it.  *amin: alpha at which the column enters.
+__device__ __forceinline__ bool cells_begin(const DevGeom &g, const RayAxis &rx, const RayAxis &ry, CellList &c,
+                                            float *amin) {
+    float lo = -FLT_MAX, hi = FLT_MAX;
+    bool miss = false;
+    clip_slab(rx, g.dx, 0, g.nx, lo, hi, miss);
+    clip_slab(ry, g.dy, 0, g.ny, lo, hi, miss);
+    if (miss || !(lo < hi)) return false;
+    const Axis ax = axis_start(rx, g.dx, lo, 0, g.nx);
+    const Axis ay = axis_start(ry, g.dy, lo, 0, g.ny);
+    c.rx = rx;
+    c.ry = ry;
+    c.rxn = ax.r;
+    c.ryn = ay.r;
+    c.sx = (float)ax.s;
+    c.sy = (float)ay.s;
+    c.ix = ax.s ? 1.0f / fabsf(g.dx * rx.I) : 0.0f;
+    c.iy = ay.s ? 1.0f / fabsf(g.dy * ry.I) : 0.0f;
+    c.col = (unsigned)zf_col(g, ax.i, ay.i);
+    c.dcx = (unsigned)(ax.s * (g.nz + 2));
+    c.dcy = (unsigned)(ay.s * g.nx * (g.nz + 2));
+    c.colmax = (unsigned)zf_col(g, g.nx - 1, g.ny - 1);
+    c.amax = hi;
+    *amin = lo;
+    return true;
+}
+
+// Writes the next cells (at most CELL_CHUNK) to `list`, padded with empty
+// cells to CELL_CHUNK, and returns their number; *last is set when the last
+// one ends at amax.  `bias` is added to every column index.  All lanes call
+// it; the values of an earlier chunk must not be in use any more.
+// The estimates of a crossing's rank are right to one: both axes' alphas carry
+// a relative rounding error of a few 2^-24 and the planes of an axis are at
+// least 1 / n of their largest alpha apart.  Column indices are clamped to the
+// volume, so that no rounding can send a load out of it.
+__device__ __forceinline__ int cells_next(const DevGeom &g, CellList &c, unsigned bias, float2 *list, bool *last) {
+    const int lane = threadIdx.x & 31;
+    constexpr float most = (float)CELL_CHUNK;
+    auto alx = [&](float m) { return c.sx != 0.0f ? plane_alpha(__fmaf_rn(c.sx, m, c.rxn), g.dx, c.rx) : FLT_MAX; };
+    auto aly = [&](float m) { return c.sy != 0.0f ? plane_alpha(__fmaf_rn(c.sy, m, c.ryn), g.dy, c.ry) : FLT_MAX; };
+    const float lf = (float)lane;
+    const float ex = alx(lf), ey = aly(lf);
+    const float ex0 = __shfl_sync(0xffffffffu, ex, 0), ey0 = __shfl_sync(0xffffffffu, ey, 0);
+    // y crossings before ex (strictly), x crossings up to ey: an x crossing
+    // comes first where both coincide
+    float ny = fminf(fmaxf(ceilf((ex - ey0) * c.iy), 0.0f), most);
+    const bool ny_high = ny > 0.0f && aly(ny - 1.0f) >= ex, ny_low = aly(ny) < ex;
+    ny = ny_high ? ny - 1.0f : ny_low ? ny + 1.0f : ny;
+    float nx = fminf(fmaxf(floorf((ey - ex0) * c.ix) + 1.0f, 0.0f), most);
+    const bool nx_high = nx > 0.0f && alx(nx - 1.0f) > ey, nx_low = alx(nx) <= ey;
+    nx = nx_high ? nx - 1.0f : nx_low ? nx + 1.0f : nx;
+    const int nxi = (int)nx, nyi = (int)ny;
+    const int rank_x = lane + nyi, rank_y = lane + nxi;
+    const unsigned cx = min(c.col + (unsigned)lane * c.dcx + (unsigned)nyi * c.dcy, c.colmax) + bias;
+    const unsigned cy = min(c.col + (unsigned)nxi * c.dcx + (unsigned)lane * c.dcy, c.colmax) + bias;
+    __syncwarp();
+    if (rank_x < CELL_CHUNK) list[rank_x] = make_float2(ex, __uint_as_float(cx));
+    if (rank_y < CELL_CHUNK) list[rank_y] = make_float2(ey, __uint_as_float(cy));
+    const int used_x = __popc(__ballot_sync(0xffffffffu, rank_x < CELL_CHUNK));
+    __syncwarp();
+    const float2 own = list[lane];
+    const int inside = __popc(__ballot_sync(0xffffffffu, own.x < c.amax));
+    const int n = min(inside + 1, CELL_CHUNK);
+    const float tail = __shfl_sync(0xffffffffu, own.y, n - 1);
+    list[lane] = make_float2(fminf(own.x, c.amax), lane < n ? own.y : tail);
+    __syncwarp();
+    c.rxn += c.sx * (float)used_x;
+    c.ryn += c.sy * (float)(CELL_CHUNK - used_x);
+    c.col += (unsigned)used_x * c.dcx + (unsigned)(CELL_CHUNK - used_x) * c.dcy;
+    *last = inside < CELL_CHUNK;
+    return n;
+}
+
 // ------------------------------------------- z index from alpha (forward)
 //
-// Along a ray the z voxel coordinate is linear in alpha: measured from the
-// plane pq nearest to the ray origin, zeta(alpha) - pq = alpha / (dz I) -
-// f / dz.  Its floor, the voxel index k, comes from one FMA and one add of
-// 1.5 * 2^23 + pq (the add rounds to an integer, and the float's bits are
-// then k + MAGIC_BITS); k - pq comes back exactly by subtracting the same
-// constant.  The alpha at which the ray leaves voxel k through a z plane is
-// (k - pq) (dz I) + c, both terms small (no cancellation).  alpha is clamped to
-// the ray's range inside [0, nz) along z, so every segment outside the volume
-// has zero length and k stays in [-1, nz].
+// Along a ray the z voxel coordinate is linear in alpha.  Measured from the
+// plane pq nearest to the ray origin, in the direction in which the ray leaves
+// the mid-plane (upwards for v > 0, downwards for v < 0: the source is at
+// z = 0, so every ray only moves away from it), it is t = a * alpha + b with
+// a >= 0.  The next plane ceil(t) comes from one add rounded up: t + m, with
+// m = 1.5 * 2^23 + c, leaves an integer whose float bits are one more than the
+// voxel index (up: c = pq) or than its mirror image (down: c = -pq), plus a
+// constant that is folded into the column's address.  The part of a cell (in
+// voxel units of z) that lies past that plane is sat(t_exit - ceil(t_entry)).
+// t is clamped to less than one voxel past the volume's end, where the padded
+// columns hold zeros.
 constexpr float ZMAGIC = 12582912.0f;        // 1.5 * 2^23
 constexpr int ZMAGIC_BITS = 0x4B400000;
 
 struct RayZ {
-    float a, b;          // (zeta - pq) - 0.5 = a * alpha + b (voxel units)
-    float m;             // ZMAGIC + pq
-    float inva, c;       // exit-plane alpha of voxel k: (k - pq) * inva + c
-    float lo, hi;        // alpha range inside the slab [0, nz)
-    int soff;            // +1 / -1 / 0: neighbour voxel across the exit plane
+    float a, b;          // t = a * alpha + b (voxel units)
+    float m;             // ZMAGIC + c
+    float hi;            // clamp of t
+    bool down;
 };
+constexpr float ZPAST = 0.99609375f;         // how far past the volume's end t may go
 
-__device__ __forceinline__ RayZ make_rayz(const RayAxis &rz, float dz, int nz) {
+// `down` is the direction to use for a ray without one of its own.
+__device__ __forceinline__ RayZ make_rayz(const RayAxis &rz, float dz, int nz, bool down) {
     RayZ r;
-    r.m = ZMAGIC + rz.pq;
-    if (rz.I == 0.0f) {                          // parallel to the z planes: fixed voxel pq
-        const bool in = rz.pq >= 0.0f && rz.pq < (float)nz;
-        r.a = r.b = r.inva = 0.0f;
-        r.c = FLT_MAX;
-        r.lo = in ? -FLT_MAX : 0.0f;
-        r.hi = in ? FLT_MAX : 0.0f;
-        r.soff = 0;
-        return r;
+    if (rz.I == 0.0f) {                          // parallel to the z planes: fixed voxel (pads: outside)
+        const float k = fminf(rz.pq, (float)nz);
+        r.a = 0.0f;
+        r.b = 0.5f;
+        r.down = down;
+        r.m = ZMAGIC + (down ? -1.0f - k : k);
+        r.hi = 0.5f + ZPAST;
+    } else {
+        r.down = rz.I < 0.0f;
+        r.a = 1.0f / fabsf(dz * rz.I);
+        const float b = rz.f / dz;
+        r.b = r.down ? b : -b;
+        r.m = ZMAGIC + (r.down ? -rz.pq : rz.pq);
+        r.hi = (r.down ? rz.pq : (float)nz - rz.pq) + ZPAST;
     }
-    const float a0 = plane_alpha(0.0f - rz.pq, dz, rz), a1 = plane_alpha((float)nz - rz.pq, dz, rz);
-    r.lo = fminf(a0, a1);
-    r.hi = fmaxf(a0, a1);
-    r.inva = dz * rz.I;
-    r.a = 1.0f / r.inva;
-    r.b = -rz.f / dz - 0.5f;
-    const bool up = rz.I > 0.0f;                 // alpha grows with the plane index
-    r.c = up ? (dz + rz.f) * rz.I : rz.f * rz.I; // exit plane of voxel k: k + 1 (up) or k (down)
-    r.soff = up ? 1 : -1;
     return r;
 }
 
-// Forward traversal of R rays of one detector column through the padded
-// z-fastest volume, for geometries with at most one z-plane crossing per xy
-// cell (DevGeom::zsingle).  At every xy cell boundary e each ray adds
-//     (e - e_prev) v + max(e - ze, 0) (vn - v),
-// v and vn the voxel it occupied on entering the cell and its neighbour across
-// the next z plane (crossed at ze if ze < e): both are loaded for every cell,
-// so no lane branches.  The next cell's voxel index comes from zeta(e).  Ray
-// pairs use packed FP32x2 arithmetic unless COMP (Kahan-compensated sums, for
-// 16-bit storage).  Returns the ray sums in acc (alpha units).
-template <typename T, bool COMP, int R>
-__device__ __forceinline__ void trace_rays_zsingle(const DevGeom &g, const T *__restrict__ vol, const RayAxis &rx,
-                                                   const RayAxis &ry, const RayAxis (&rzax)[R], float (&acc)[R]) {
-    const int nx = g.nx, ny = g.ny, nz = g.nz;
-    float amin = -FLT_MAX, amax = FLT_MAX;
-    bool miss = false;
-    clip_slab(rx, g.dx, 0, nx, amin, amax, miss);
-    clip_slab(ry, g.dy, 0, ny, amin, amax, miss);
-    if (miss || !(amin < amax)) return;
-    Axis ax = axis_start(rx, g.dx, amin, 0, nx);
-    Axis ay = axis_start(ry, g.dy, amin, 0, ny);
-    const int sx = nz + 2, sy = nx * (nz + 2);
-    // index of voxel k of the current column is base + bits(k + ZMAGIC)
-    int base = (int)zf_col(g, ax.i, ay.i) - ZMAGIC_BITS;
-    RayZ z[R];
-    float kf[R], v[R], vn[R], ep[R], comp[R];
-    auto ld = [&](int idx) { return Storage<T>::load(vol + idx); };
+// Walks R rays of one detector column through the padded z-fastest volume, for
+// geometries with at most one z-plane crossing per xy cell
+// (DevGeom::zsingle).  In every cell of alpha length L a ray adds
+//     L v + (part past the next plane) (vn - v),
+// v and vn the voxel it entered the cell in and its neighbour across that
+// plane: both are loaded for every cell (one address, the neighbour at a fixed
+// offset), so no lane branches.  DIR: +1 / -1 when every ray of the warp goes
+// up / down, 0 when both occur (the row group around the mid-plane); CLAMP:
+// some ray leaves the volume through its top or bottom.  OFF32: the padded volume
+// has at most 2^32 bytes (OFF32_BYTES), so a voxel's address is one 32-bit
+// multiply-add from the volume's base instead of a 64-bit one.  Ray pairs use packed
+// FP32x2 arithmetic.  The sums of a chunk of cells are folded into acc (with
+// Kahan compensation for 16-bit storage, COMP) every CELL_CHUNK cells.
+// Returns the ray sums in acc (alpha units).
+// A x at 256^3 / 512^2 / 360 angles: 24.2 -> 12.9 ms, 24 -> 12.6 warp
+// instructions per cell and 32 rays (two loads, one and a half packed FMA
+// pairs and an add for the sums, two for t and the plane, the rest address and
+// list), issue slots 62 % busy and L1 data wavefronts 54 %.
+template <typename T, bool COMP, int R, bool OFF32, int DIR, bool CLAMP>
+__device__ __forceinline__ void walk_cells(const DevGeom &g, const T *__restrict__ vol, CellList &cl, float amin,
+                                           const RayZ (&z)[R], float4 *list, float (&acc)[R]) {
+    constexpr int UNR = R == 2 ? 8 : 4;          // cells whose loads are in flight together
+    float kb[R], kf[R], comp[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        z[r] = make_rayz(rzax[r], g.dz, nz);
-        ep[r] = fminf(fmaxf(amin, z[r].lo), z[r].hi);
-        const float kb = __fadd_rn(__fmaf_rn(ep[r], z[r].a, z[r].b), z[r].m);
-        kf[r] = __fadd_rn(kb, -z[r].m);
-        const int idx = base + __float_as_int(kb);
-        v[r] = ld(idx);
-        vn[r] = ld(idx + z[r].soff);
+        float t = __fmaf_rn(amin, z[r].a, z[r].b);
+        if (CLAMP) t = fminf(t, z[r].hi);
+        kb[r] = __fadd_ru(t, z[r].m);
+        kf[r] = kb[r] - z[r].m;
         comp[r] = 0.0f;
     }
-    auto kahan = [&](int r, float term) {
-        const float yk = term - comp[r];
-        const float t = acc[r] + yk;
-        comp[r] = (t - acc[r]) - yk;
-        acc[r] = t;
-    };
-    const int dcx = ax.s * sx, dcy = ay.s * sy;
-    const int maxsteps = nx + ny + 1;
+    float ep = amin;
+    bool last = false;
+    const int maxchunks = (g.nx + g.ny) / CELL_CHUNK + 2;
+    // voxel index k of the column: col - 1 + (bits(kb) - ZMAGIC_BITS) (up),
+    // col - (bits(kb) - ZMAGIC_BITS) (down); the constant is added in the list
+    constexpr unsigned UP = 0u - (unsigned)ZMAGIC_BITS - 1u, DOWN = (unsigned)ZMAGIC_BITS;
 #pragma unroll 1
-    for (int n = 0; n < maxsteps; ++n) {
-        const float e = fminf(ax.e, ay.e);
-        float kbn[R];
-        if (!COMP && R % 2 == 0) {
+    for (int chunk = 0; chunk < maxchunks && !last; ++chunk) {
+        const int n = cells_next(g, cl, DIR > 0 ? UP : DIR < 0 ? DOWN : 0u, (float2 *)list, &last);
+        float s1[R], s2[R];
 #pragma unroll
-            for (int p = 0; p < R / 2; ++p) {
-                const int r0 = 2 * p, r1 = r0 + 1;
-                const float2 ec = make_float2(fminf(fmaxf(e, z[r0].lo), z[r0].hi), fminf(fmaxf(e, z[r1].lo), z[r1].hi));
-                const float2 len = __fadd2_rn(ec, make_float2(-ep[r0], -ep[r1]));
-                float2 a2 = __ffma2_rn(len, make_float2(v[r0], v[r1]), make_float2(acc[r0], acc[r1]));
-                const float2 ze = __ffma2_rn(make_float2(kf[r0], kf[r1]), make_float2(z[r0].inva, z[r1].inva),
-                                             make_float2(z[r0].c, z[r1].c));
-                const float2 d = __fadd2_rn(ec, make_float2(-ze.x, -ze.y));
-                const float2 w = make_float2(fmaxf(d.x, 0.0f), fmaxf(d.y, 0.0f));
-                const float2 dv = __fadd2_rn(make_float2(vn[r0], vn[r1]), make_float2(-v[r0], -v[r1]));
-                a2 = __ffma2_rn(w, dv, a2);
-                acc[r0] = a2.x;
-                acc[r1] = a2.y;
-                const float2 t = __ffma2_rn(ec, make_float2(z[r0].a, z[r1].a), make_float2(z[r0].b, z[r1].b));
-                const float2 kb = __fadd2_rn(t, make_float2(z[r0].m, z[r1].m));
-                const float2 kn = __fadd2_rn(kb, make_float2(-z[r0].m, -z[r1].m));
-                kbn[r0] = kb.x;
-                kbn[r1] = kb.y;
-                kf[r0] = kn.x;
-                kf[r1] = kn.y;
-                ep[r0] = ec.x;
-                ep[r1] = ec.y;
+        for (int r = 0; r < R; ++r) s1[r] = s2[r] = 0.0f;
+#pragma unroll 1
+        for (int c0 = 0; c0 < n; c0 += UNR) {
+            float e[UNR];
+            unsigned col[UNR];
+#pragma unroll
+            for (int p = 0; p < UNR / 2; ++p) {
+                const float4 c2 = list[c0 / 2 + p];
+                e[2 * p] = c2.x;
+                col[2 * p] = __float_as_uint(c2.y);
+                e[2 * p + 1] = c2.z;
+                col[2 * p + 1] = __float_as_uint(c2.w);
             }
-        } else {
+            float v[UNR][R], vn[UNR][R], w[UNR][R], len[UNR];
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const float ec = fminf(fmaxf(e, z[r].lo), z[r].hi);
-                const float ze = __fmaf_rn(kf[r], z[r].inva, z[r].c);
-                const float w = fmaxf(ec - ze, 0.0f);
-                if (COMP) {
-                    kahan(r, (ec - ep[r]) * v[r]);
-                    kahan(r, w * (vn[r] - v[r]));
-                } else {
-                    acc[r] = __fmaf_rn(ec - ep[r], v[r], acc[r]);
-                    acc[r] = __fmaf_rn(w, vn[r] - v[r], acc[r]);
+            for (int u = 0; u < UNR; ++u) {
+                // DOWN + col stays below 2^32, so it is zero-extended; UP + col wraps to a negative index
+                const T *base = DIR > 0 ? vol + (int64_t)(int)col[u] : vol + (int64_t)col[u];
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int bits = __float_as_int(kb[r]);
+                    const int step = DIR != 0 ? DIR : z[r].down ? -1 : 1;
+                    const T *ptr;
+                    if (OFF32) {
+                        const unsigned c = DIR == 0 ? col[u] + (z[r].down ? DOWN : UP) : col[u];
+                        ptr = (const T *)((const char *)vol + (size_t)((c + (unsigned)bits * (unsigned)step) * (unsigned)sizeof(T)));
+                    } else {
+                        ptr = base + (int64_t)bits * step;
+                        if (DIR == 0) ptr += z[r].down ? (int64_t)ZMAGIC_BITS : -(int64_t)ZMAGIC_BITS - 1;
+                    }
+                    v[u][r] = Storage<T>::load(ptr);
+                    vn[u][r] = Storage<T>::load(ptr + step);
                 }
-                const float kb = __fadd_rn(__fmaf_rn(ec, z[r].a, z[r].b), z[r].m);
-                kf[r] = __fadd_rn(kb, -z[r].m);
-                kbn[r] = kb;
-                ep[r] = ec;
+                len[u] = e[u] - ep;
+                ep = e[u];
+                const float2 e2 = make_float2(e[u], e[u]);
+                if (R % 2 == 0) {
+#pragma unroll
+                    for (int r = 0; r + 1 < R; r += 2) {
+                        float2 t = __ffma2_rn(e2, make_float2(z[r].a, z[r + 1].a), make_float2(z[r].b, z[r + 1].b));
+                        if (CLAMP) t = make_float2(fminf(t.x, z[r].hi), fminf(t.y, z[r + 1].hi));
+                        w[u][r] = __saturatef(t.x - kf[r]);
+                        w[u][r + 1] = __saturatef(t.y - kf[r + 1]);
+                        const float2 m2 = make_float2(z[r].m, z[r + 1].m);
+                        const float2 k2 = __fadd2_ru(t, m2);
+                        const float2 f2 = __ffma2_rn(m2, make_float2(-1.0f, -1.0f), k2);
+                        kb[r] = k2.x;
+                        kb[r + 1] = k2.y;
+                        kf[r] = f2.x;
+                        kf[r + 1] = f2.y;
+                    }
+                } else {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        float t = __fmaf_rn(e[u], z[r].a, z[r].b);
+                        if (CLAMP) t = fminf(t, z[r].hi);
+                        w[u][r] = __saturatef(t - kf[r]);
+                        kb[r] = __fadd_ru(t, z[r].m);
+                        kf[r] = kb[r] - z[r].m;
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < UNR; ++u) {
+                if (R % 2 == 0) {
+                    const float2 l2 = make_float2(len[u], len[u]);
+#pragma unroll
+                    for (int r = 0; r + 1 < R; r += 2) {
+                        const float2 v2 = make_float2(v[u][r], v[u][r + 1]);
+                        const float2 d2 = __ffma2_rn(v2, make_float2(-1.0f, -1.0f), make_float2(vn[u][r], vn[u][r + 1]));
+                        const float2 a1 = __ffma2_rn(l2, v2, make_float2(s1[r], s1[r + 1]));
+                        const float2 a2 = __ffma2_rn(make_float2(w[u][r], w[u][r + 1]), d2, make_float2(s2[r], s2[r + 1]));
+                        s1[r] = a1.x;
+                        s1[r + 1] = a1.y;
+                        s2[r] = a2.x;
+                        s2[r + 1] = a2.y;
+                    }
+                } else {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        s1[r] = __fmaf_rn(len[u], v[u][r], s1[r]);
+                        s2[r] = __fmaf_rn(w[u][r], vn[u][r] - v[u][r], s2[r]);
+                    }
+                }
             }
         }
-        bool done;
-        if (e == ax.e) {
-            ax.i += ax.s;
-            done = (unsigned)ax.i >= (unsigned)nx;
-            if (!done) {
-                base += dcx;
-                ax.r += (float)ax.s;
-                ax.e = plane_alpha(ax.r, g.dx, rx);
-            }
-        } else {
-            ay.i += ay.s;
-            done = (unsigned)ay.i >= (unsigned)ny;
-            if (!done) {
-                base += dcy;
-                ay.r += (float)ay.s;
-                ay.e = plane_alpha(ay.r, g.dy, ry);
-            }
-        }
-        if (done) break;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            const int idx = base + __float_as_int(kbn[r]);
-            v[r] = ld(idx);
-            vn[r] = ld(idx + z[r].soff);
+            // alpha per voxel: 1 / a (no ray parallel to the z planes has an s2)
+            const float term = z[r].a > 0.0f ? s1[r] + __fdividef(s2[r], z[r].a) : s1[r];
+            if (COMP) {
+                const float yk = term - comp[r];
+                const float t = acc[r] + yk;
+                comp[r] = (t - acc[r]) - yk;
+                acc[r] = t;
+            } else {
+                acc[r] += term;
+            }
         }
     }
+}
+
+// Forward traversal of R rays of one detector column (DevGeom::zsingle):
+// the walk for the warp's directions and z range.  list: 2 * CELL_CHUNK floats
+// of shared memory of this warp.
+template <typename T, bool COMP, int R, bool OFF32>
+__device__ __forceinline__ void trace_rays_zsingle(const DevGeom &g, const T *__restrict__ vol, const RayAxis &rx,
+                                                   const RayAxis &ry, const RayAxis (&rzax)[R], float4 *list,
+                                                   float (&acc)[R]) {
+    CellList cl;
+    float amin;
+    if (!cells_begin(g, rx, ry, cl, &amin)) return;
+    bool up = false, down = false;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        up = up || rzax[r].I > 0.0f;
+        down = down || rzax[r].I < 0.0f;
+    }
+    up = __any_sync(0xffffffffu, up);
+    down = __any_sync(0xffffffffu, down);
+    RayZ z[R];
+    bool inside = true;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        z[r] = make_rayz(rzax[r], g.dz, g.nz, down && !up);
+        inside = inside && __fmaf_rn(cl.amax, z[r].a, z[r].b) <= z[r].hi - ZPAST;
+    }
+    inside = __all_sync(0xffffffffu, inside);
+    if (up && down)
+        walk_cells<T, COMP, R, OFF32, 0, true>(g, vol, cl, amin, z, list, acc);
+    else if (!down)
+        inside ? walk_cells<T, COMP, R, OFF32, 1, false>(g, vol, cl, amin, z, list, acc)
+               : walk_cells<T, COMP, R, OFF32, 1, true>(g, vol, cl, amin, z, list, acc);
+    else
+        inside ? walk_cells<T, COMP, R, OFF32, -1, false>(g, vol, cl, amin, z, list, acc)
+               : walk_cells<T, COMP, R, OFF32, -1, true>(g, vol, cl, amin, z, list, acc);
 }
 
 // ------------------------------------------------------------- forward A x
@@ -402,12 +559,15 @@ __device__ __forceinline__ void trace_rays_zsingle(const DevGeom &g, const T *__
 // through the traversal, and the sums need no block barrier (measured 6 %
 // of the transpose's time with one).
 
-constexpr int FWD_COLS = 8, FWD_THREADS = 32 * FWD_COLS;
+// lists: FWD_COLS * FWD_LIST float4 of shared memory (the warps' cell lists).
 
-template <typename T, bool COMP, int R, bool VFAST, typename PartialAt>
+constexpr int FWD_COLS = 8, FWD_THREADS = 32 * FWD_COLS;
+constexpr int FWD_LIST = CELL_CHUNK / 2;         // float4 of one warp's cell list
+
+template <typename T, bool COMP, int R, bool VFAST, bool OFF32, typename PartialAt>
 __device__ __forceinline__ void forward_tile(const DevGeom &g, const T *__restrict__ vol, T *__restrict__ proj,
                                              const Epilogue &epi, int tx, int ty, int a, PartialAt &&partial_at,
-                                             double *red) {
+                                             float4 *lists) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int iu = tx * FWD_COLS + warp;
     const int iv0 = ty * 32 * R;
@@ -419,7 +579,7 @@ __device__ __forceinline__ void forward_tile(const DevGeom &g, const T *__restri
         RayAxis rx, ry, rz[R];
         load_rays<R>(g, a, iu, iv0, g.nv, rx, ry, rz);
         if (g.zsingle) {
-            trace_rays_zsingle<T, COMP, R>(g, vol, rx, ry, rz, acc);
+            trace_rays_zsingle<T, COMP, R, OFF32>(g, vol, rx, ry, rz, lists + warp * FWD_LIST, acc);
         } else {
             // several z crossings per xy cell are possible: the exact
             // crossing-by-crossing traversal

@@ -52,7 +52,7 @@ struct SlotDev {
     const double *qf, *qb;  // the partials the scalar steps read: pf / pb, or their folds
     int nqf, nqb;
     int method, cap;
-    int fgx, fgy;          // forward tile grid (x: columns / 8, y: row groups); z: angles
+    int fgx;               // forward tiles along x (columns / 8); then angles, then row groups
     int bgx, bgy;          // brick grid (x, y); z: bricks along z
     int64_t m;             // length of a volume-side vector (padded z-fastest layout)
 };
@@ -97,8 +97,8 @@ static_assert(sizeof(DevGeom) % sizeof(int) == 0 && sizeof(DevGeom) / sizeof(int
               "DevGeom is copied one int per thread");
 
 // U <- fa * A V + fb * U for every slot (forward tiles of all slots).
-__global__ void __launch_bounds__(FWD_THREADS, 3) srv_forward(const SlotTable *tab, unsigned *counter) {
-    __shared__ double red[FWD_THREADS / 32];
+__global__ void __launch_bounds__(FWD_THREADS, 2) srv_forward(const SlotTable *tab, unsigned *counter) {
+    __shared__ float4 lists[FWD_COLS * FWD_LIST];
     __shared__ int item_sh;
     __shared__ DevGeom g_sh;               // the claimed tile's geometry
     const int n = tab->n;
@@ -110,10 +110,10 @@ __global__ void __launch_bounds__(FWD_THREADS, 3) srv_forward(const SlotTable *t
         if (threadIdx.x < sizeof(DevGeom) / sizeof(int)) ((int *)&g_sh)[threadIdx.x] = ((const int *)&sd.g)[threadIdx.x];
         __syncthreads();
         const int local = item - tab->fwd_start[s];
-        const int tx = local % sd.fgx, ty = (local / sd.fgx) % sd.fgy, a = local / (sd.fgx * sd.fgy);
+        const int tx = local % sd.fgx, a = (local / sd.fgx) % g_sh.nangles, ty = local / (sd.fgx * g_sh.nangles);   // as forward_grid
         const Epilogue epi{&sd.st->fa, &sd.st->fb, 0.0, 0.0, nullptr, nullptr, nullptr, sd.Uw};
-        forward_tile<float, false, SRV_FWD_ROWS, true>(g_sh, sd.V, sd.U, epi, tx, ty, a,
-                                                       [&]() { return sd.pf + (size_t)local * TILE_PARTIALS; }, red);
+        forward_tile<float, false, SRV_FWD_ROWS, true, false>(g_sh, sd.V, sd.U, epi, tx, ty, a,
+                                                       [&]() { return sd.pf + (size_t)local * TILE_PARTIALS; }, lists);
     }
 }
 
@@ -679,7 +679,7 @@ void ServerImpl::run_steps() {
                 d.method = sl.req->method;
                 d.cap = sl.req->iters;
                 const dim3 fg = forward_grid(d.g), bg = backward_grid(d.g);
-                d.fgx = fg.x; d.fgy = fg.y; d.bgx = bg.x; d.bgy = bg.y;
+                d.fgx = fg.x; d.bgx = bg.x; d.bgy = bg.y;
                 d.m = zf_len(d.g);
                 t.fwd_start[i + 1] = t.fwd_start[i] + sl.nf;
                 t.bwd_start[i + 1] = t.bwd_start[i] + sl.nb;
