@@ -50,14 +50,16 @@ struct DevGeom {
     const float2 *zbox;      // [nz][nv]: alpha interval (entry, exit) of row iv's ray in z slab k
     int zsingle;             // 1: every ray crosses at most one z plane inside any x/y voxel column
     int fwd_rows;            // forward tile: rays per lane (1, 2 or 4)
-    int bwd_config;          // transpose tile: column patch / voxels per lane (backward_shape)
+    int bwd_config;          // transpose tile (backward_shape)
+    int patch_columns;       // patch tile: most detector columns across a patch, 0 when it does not apply
+    float rho, rho_hi, rho_lo;   // dz / dv, and its leading 11 bits and the rest
+    float m_hi, m_lo;        // the same for dso / dsd
     int angle_block;         // transpose: angles per pass when summed in passes (launch_backward)
 };
 
-// Tile of the transpose: a bx x by patch of voxel columns (one warp each),
-// bz = 32 r voxels along z (r per lane).
+// Tile of the transpose: bx x by voxel columns, bz voxels along z.
 struct BrickShape {
-    int bx, by, bz, r;
+    int bx, by, bz;
 };
 
 // ------------------------------------------------- internal volume layout
@@ -232,7 +234,9 @@ inline int forward_num_partials(const DevGeom &g) { return forward_num_blocks(g)
 inline int backward_num_partials(const DevGeom &g) { return backward_num_blocks(g) * TILE_PARTIALS; }
 dim3 forward_grid(const DevGeom &g);
 dim3 backward_grid(const DevGeom &g);
-BrickShape backward_shape(int config);
+BrickShape backward_shape(const DevGeom &g);
+// Whether the geometry's configuration runs as patch tiles (patch_tile.cuh).
+bool backward_patches(const DevGeom &g);
 constexpr int NUM_FWD_ROWS = 3, NUM_BWD_CONFIGS = 10;
 
 }  // namespace cbct

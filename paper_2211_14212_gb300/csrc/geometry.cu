@@ -107,6 +107,41 @@ cbct_status validate_geometry_desc(const cbct_geometry_desc *d) {
 // (cbct_geometry_set_angle_block).
 namespace cbct {
 int default_angle_block(const DevGeom &g) { return g.nangles; }
+
+// v's leading 11 bits
+static float leading(double v) {
+    int e = 0;
+    const double f = std::frexp(v, &e);
+    return (float)std::ldexp(std::nearbyint(f * 2048.0), e - 11);
+}
+
+// Where the patch tile applies (patch_tile.cuh), and its constants: bounds of
+// a patch's footprint over every position and angle.
+static void set_patch_bounds(DevGeom &g, const cbct_geometry_desc &d) {
+    const double rho = d.dz / d.dv, m = d.dso / d.dsd;
+    g.rho = (float)rho;
+    g.rho_hi = leading(rho);
+    g.rho_lo = (float)(rho - g.rho_hi);
+    g.m_hi = leading(m);
+    g.m_lo = (float)(m - g.m_hi);
+    g.patch_columns = 0;
+    // a patch may reach one voxel out of the volume
+    const double r = std::hypot((0.5 * d.nx + 1.0) * d.dx, (0.5 * d.ny + 1.0) * d.dy);
+    if (r >= 0.95 * d.dso) return;
+    const double diagonal = 2.0 * std::hypot(d.dx, d.dy);
+    const double near = d.dsd / (d.dso - r), far = d.dsd / (d.dso + r);     // magnifications
+    const double fan = d.dso / std::sqrt(d.dso * d.dso - r * r);            // 1 / cos of the fan's half angle
+    const double columns = std::ceil(diagonal * near * fan / d.du + 0.2) + 1.0;
+    // rows a plane passes between a patch's near and far depth, at the volume's end
+    const double passed = 0.5 * d.nz * rho * near * diagonal / (d.dso - r);
+    // half integers of 12 bits times 11 bits are exact (patch_crossing); a
+    // slab covers more than the margins of its planes; 32-bit offsets within
+    // a projection; the lists fit 48 KB of shared memory
+    if (columns > 22.0 || passed + 2.0 * 0.05 > 1.95 || rho * far < 0.25 || d.nz > 4096 || d.nv > 4096 || d.nv < 3 ||
+        (int64_t)d.nu * d.nv >= (int64_t)1 << 30)
+        return;
+    g.patch_columns = std::max(4, (int)columns);
+}
 }  // namespace cbct
 
 extern "C" cbct_status cbct_geometry_create(const cbct_geometry_desc *d, cbct_geometry **out) {
@@ -206,7 +241,11 @@ extern "C" cbct_status cbct_geometry_create(const cbct_geometry_desc *d, cbct_ge
         const double zrise = std::sqrt(d->dx * d->dx + d->dy * d->dy) * vmax / d->dsd;
         dg.zsingle = zrise < 0.98 * d->dz ? 1 : 0;
     }
-    dg.bwd_config = nz >= 64 ? 3 : 0;   // 2 / 1 voxels per lane by column depth
+    set_patch_bounds(dg, *d);
+    if (dg.patch_columns > 0 && nz > 64)
+        dg.bwd_config = nz > 128 ? 7 : 5;   // patch tiles of 256 / 128 voxels along z
+    else
+        dg.bwd_config = nz >= 64 ? 3 : 0;   // 2 / 1 voxels per lane by column depth
     dg.angle_block = default_angle_block(dg);
     *out = g;
     return CBCT_OK;

@@ -125,26 +125,28 @@ cbct_status launch_count(const DevGeom &g, unsigned long long *count_dev, cudaSt
 
 // ---------------------------------------------------------- transpose A^T y
 
-// Transpose tile shapes: column patch CX x (8 / CX), 32 K voxels along z;
-// configurations 0..3 and 8, 9 keep the slab intervals of their candidate
-// rows in registers per angle (8, 9: 4 voxels per lane, 3 CTAs per SM).
-BrickShape backward_shape(int config) {
-    switch (config) {
-    case 8: return BrickShape{2, 4, 128, 4};
-    case 9: return BrickShape{4, 2, 128, 4};
-    case 1: return BrickShape{4, 2, 64, 2};
-    case 2: return BrickShape{8, 1, 32, 1};
-    case 3: return BrickShape{2, 4, 64, 2};
-    case 4: return BrickShape{4, 2, 128, 4};
-    case 5: return BrickShape{2, 4, 128, 4};
-    case 6: return BrickShape{4, 2, 256, 8};
-    case 7: return BrickShape{2, 4, 256, 8};
-    default: return BrickShape{4, 2, 32, 1};
+// Transpose tile shapes.  4..7 are patch tiles where the geometry allows them
+// (DevGeom::patch_columns) and the 4-voxel tiles 9 and 8 elsewhere.
+bool backward_patches(const DevGeom &g) { return g.patch_columns > 0 && g.bwd_config >= 4 && g.bwd_config <= 7; }
+
+BrickShape backward_shape(const DevGeom &g) {
+    const bool patches = backward_patches(g);
+    switch (g.bwd_config) {
+    case 1: return BrickShape{4, 2, 64};
+    case 2: return BrickShape{8, 1, 32};
+    case 3: return BrickShape{2, 4, 64};
+    case 4: return BrickShape{4, 2, 128};
+    case 5: return BrickShape{2, 4, 128};
+    case 6: return BrickShape{4, 2, patches ? 256 : 128};
+    case 7: return BrickShape{2, 4, patches ? 256 : 128};
+    case 8: return BrickShape{2, 4, 128};
+    case 9: return BrickShape{4, 2, 128};
+    default: return BrickShape{4, 2, 32};
     }
 }
 
 dim3 backward_grid(const DevGeom &g) {
-    const BrickShape b = backward_shape(g.bwd_config);
+    const BrickShape b = backward_shape(g);
     return dim3((g.nx + b.bx - 1) / b.bx, (g.ny + b.by - 1) / b.by, (g.nz + b.bz - 1) / b.bz);
 }
 

@@ -692,7 +692,6 @@ __device__ __forceinline__ void for_crossing_columns(const DevGeom &g, int a, in
         }
     }
 }
-constexpr int BWD_SHORT_ROWS = 3;
 
 // Angles [a_begin, a_end) are summed in one call.  A scan whose projections
 // do not fit in L2 is summed in passes over blocks of angles (launch_backward):
@@ -704,20 +703,18 @@ constexpr int BWD_SHORT_ROWS = 3;
 // ((j * nx + i) * nz + k) (unpadded); they may be the same buffer (each lane
 // reads and writes only its own voxels).  ZFAST output goes to the padded
 // z-fastest layout, else to the ABI layout x[k][j][i].
-template <typename T, bool ZFAST, int CX, int K, bool HOIST, int IU_UNROLL = 0, typename PartialAt>
+template <typename T, bool ZFAST, int CX, int K, int IU_UNROLL = 0, typename PartialAt>
 __device__ __forceinline__ void backward_tile(const DevGeom &g, const float *__restrict__ wproj, T *__restrict__ vol,
                                               const Epilogue &epi, int tx, int ty, int tz, int a_begin, int a_end,
-                                              const float *acc_in, float *acc_out, PartialAt &&partial_at,
-                                              double *red) {
+                                              const float *acc_in, float *acc_out, PartialAt &&partial_at) {
     constexpr int CY = 8 / CX;
     // detector columns clipped by the lanes at once (tiles of up to 2 voxels
     // per lane; the 4-voxel tiles keep the per-column clip, which needs fewer
     // registers) and columns per unrolled step of the column loops
     constexpr bool BWD_LANE_CLIP = K <= 2;
-    constexpr int BWD_IU_UNROLL = IU_UNROLL > 0 ? IU_UNROLL : !HOIST ? 1 : K == 1 ? 2 : K == 2 ? 1 : 2;
-    // HOIST: the slab intervals of the candidate rows are loaded once per
-    // angle and kept in registers (2 or 3 rows x 2 floats per voxel of the
-    // lane); otherwise they are loaded for every detector column.
+    constexpr int BWD_IU_UNROLL = IU_UNROLL > 0 ? IU_UNROLL : K == 2 ? 1 : 2;
+    // The slab intervals of the candidate rows are loaded once per angle and
+    // kept in registers (2 or 3 rows x 2 floats per voxel of the lane).
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i = tx * CX + (warp % CX), j = ty * CY + (warp / CX);
     const int k0 = tz * 32 * K;
@@ -728,7 +725,7 @@ __device__ __forceinline__ void backward_tile(const DevGeom &g, const float *__r
         const int k = k0 + kk * 32 + lane;
         acc[kk] = acc_in && col_ok && k < g.nz ? acc_in[((size_t)j * g.nx + i) * g.nz + k] : 0.0f;
     }
-    if (col_ok && HOIST) {
+    if (col_ok) {
         // The three candidate rows of each voxel start at its window's first
         // row moved down to fit the detector, and their slab intervals are
         // loaded once per angle (a row outside the window meets the voxel
@@ -841,89 +838,6 @@ __device__ __forceinline__ void backward_tile(const DevGeom &g, const float *__r
                     }
                 });
             }
-        }
-    }
-    if (col_ok && !HOIST) {
-        const float x0 = g.bx0 + i * g.dx, x1 = x0 + g.dx;
-        const float y0 = g.by0 + j * g.dy, y1 = y0 + g.dy;
-        const float cu = 0.5f * (g.nu - 1), cv = 0.5f * (g.nv - 1);
-        // The detector windows below only select candidates (every length is
-        // then computed exactly from plane_alpha), so they use fast
-        // approximate divisions: their relative error (~1e-6) stays far below
-        // the 0.05-pixel margins.
-        const float inv_du = 1.0f / g.du, inv_dv = 1.0f / g.dv;
-        const size_t nuv = (size_t)g.nu * g.nv;
-        for (int a = a_begin; a < a_end; ++a) {
-            const float2 cs = __ldg(&g.trig[a]);
-            float umin = FLT_MAX, umax = -FLT_MAX, magmin = FLT_MAX, magmax = 0.0f;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const float px = (c & 1) ? x1 : x0, py = (c & 2) ? y1 : y0;
-                const float along = g.dso - (px * cs.x + py * cs.y);   // > 0: source outside
-                const float mag = __fdividef(g.dsd, along);
-                const float u = (-px * cs.y + py * cs.x) * mag;
-                umin = fminf(umin, u);
-                umax = fmaxf(umax, u);
-                magmin = fminf(magmin, mag);
-                magmax = fmaxf(magmax, mag);
-            }
-            const int iu0 = max(0, (int)ceilf(__fmaf_rn(umin, inv_du, cu - 0.05f)));
-            const int iu1 = min(g.nu - 1, (int)floorf(__fmaf_rn(umax, inv_du, cu + 0.05f)));
-            // Rows that can meet the lane's voxel at this angle: a point at
-            // height z and source depth `along` lies on row v = z dsd / along,
-            // and the column's depths span the corners' (mag = dsd / along is
-            // extreme at a corner).  The window holds for every detector
-            // column below; a row that misses the voxel for one of them adds
-            // an exact zero.
-            int r0[K], r1[K];
-#pragma unroll
-            for (int kk = 0; kk < K; ++kk) {
-                const int k = k0 + kk * 32 + lane;
-                const float zlo = (g.bz0 + k * g.dz) * inv_dv, zhi = (g.bz0 + (k + 1) * g.dz) * inv_dv;
-                const float vmin = fminf(zlo * magmin, zlo * magmax);
-                const float vmax = fmaxf(zhi * magmin, zhi * magmax);
-                r0[kk] = max(0, (int)ceilf(vmin + (cv - 0.05f)));
-                r1[kk] = k < g.nz ? min(g.nv - 1, (int)floorf(vmax + (cv + 0.05f))) : -1;
-            }
-            // Windows of at most BWD_SHORT_ROWS rows in every lane (the usual
-            // case: a slab spans dz * mag / dv rows) take a fixed, predicated
-            // sequence instead of a loop; the same rows are summed in the same
-            // order either way.
-            bool short_rows = true;
-#pragma unroll
-            for (int kk = 0; kk < K; ++kk) short_rows = short_rows && r1[kk] - r0[kk] < BWD_SHORT_ROWS;
-            short_rows = __all_sync(0xffffffffu, short_rows);
-            const float *pa = wproj + (size_t)a * nuv;
-            // unrolled by BWD_IU_UNROLL, as the hoisted walk above
-            for_crossing_columns<BWD_LANE_CLIP, BWD_IU_UNROLL>(g, a, i, j, iu0, iu1, lane, [&](int iu, float ain, float aout) {
-                const float *wcol = pa + (size_t)iu * g.nv;
-                if (short_rows) {
-#pragma unroll
-                    for (int kk = 0; kk < K; ++kk) {
-                        const float2 *zb = g.zbox + (size_t)(k0 + kk * 32 + lane) * g.nv;
-#pragma unroll
-                        for (int t = 0; t < BWD_SHORT_ROWS; ++t) {
-                            const int iv = r0[kk] + t;
-                            if (iv <= r1[kk]) {
-                                const float2 e = __ldg(zb + iv);
-                                const float lo = fmaxf(ain, e.x), hi = fminf(aout, e.y);
-                                acc[kk] = __fmaf_rn(fmaxf(hi - lo, 0.0f), __ldg(wcol + iv), acc[kk]);
-                            }
-                        }
-                    }
-                } else {
-#pragma unroll
-                    for (int kk = 0; kk < K; ++kk) {
-                        const float2 *zb = g.zbox + (size_t)(k0 + kk * 32 + lane) * g.nv;
-                        for (int iv = r0[kk]; iv <= r1[kk]; ++iv) {
-                            const float2 e = __ldg(zb + iv);        // row iv's alpha interval in slab k
-                            const float lo = fmaxf(ain, e.x), hi = fminf(aout, e.y);
-                            // a miss adds exactly zero: the same sum as skipping it
-                            acc[kk] = __fmaf_rn(fmaxf(hi - lo, 0.0f), __ldg(wcol + iv), acc[kk]);
-                        }
-                    }
-                }
-            });
         }
     }
     if (acc_out) {                      // an earlier pass: keep the running sums

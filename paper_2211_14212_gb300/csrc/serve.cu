@@ -119,7 +119,6 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) srv_forward(const SlotTable *t
 
 // V <- ba * A^T U + bb * V for every slot (transpose tiles of all slots, z-fastest volumes).
 __global__ void __launch_bounds__(BWD_THREADS, 4) srv_backward(const SlotTable *tab, unsigned *counter) {
-    __shared__ double red[BWD_THREADS / 32];
     __shared__ int item_sh;
     __shared__ DevGeom g_sh;               // the claimed tile's geometry
     const int n = tab->n;
@@ -133,9 +132,9 @@ __global__ void __launch_bounds__(BWD_THREADS, 4) srv_backward(const SlotTable *
         const int local = item - tab->bwd_start[s];
         const int tbx = local % sd.bgx, tby = (local / sd.bgx) % sd.bgy, tbz = local / (sd.bgx * sd.bgy);
         const Epilogue epi{&sd.st->ba, &sd.st->bb, 0.0, 0.0, nullptr, nullptr, nullptr};
-        backward_tile<float, true, SRV_CX, SRV_BK, true, 2>(g_sh, sd.Uw, sd.V, epi, tbx, tby, tbz, 0, g_sh.nangles,
+        backward_tile<float, true, SRV_CX, SRV_BK, 2>(g_sh, sd.Uw, sd.V, epi, tbx, tby, tbz, 0, g_sh.nangles,
                                                          nullptr, nullptr,
-                                                         [&]() { return sd.pb + (size_t)local * TILE_PARTIALS; }, red);
+                                                         [&]() { return sd.pb + (size_t)local * TILE_PARTIALS; });
     }
 }
 

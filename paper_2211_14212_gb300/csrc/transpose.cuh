@@ -10,29 +10,47 @@
 // the running-sum buffers (fewer live registers through the angle loop).
 #pragma once
 
-#include "projector_device.cuh"
+#include "patch_tile.cuh"
 
 namespace cbct {
 
-// Hoisted tiles of 2 or 4 voxels per lane and 8-voxel tiles run 3 CTAs per
-// SM (80 registers): the 2-voxel tiles clip their detector columns across the
-// lanes, which measured 36.6 ms at 256^3 this way against 39.0 ms at 4 CTAs.
-template <typename T, bool ZFAST, int CX, int K, bool HOIST, bool PASSES>
-__global__ void __launch_bounds__(BWD_THREADS, (K >= 8 || (HOIST && K >= 2)) ? 3 : 4)
+// Tiles of 2 or 4 voxels per lane run 3 CTAs per SM (80 registers): the
+// 2-voxel tiles clip their detector columns across the lanes, which measured
+// 36.6 ms at 256^3 this way against 39.0 ms at 4 CTAs.
+template <typename T, bool ZFAST, int CX, int K, bool PASSES>
+__global__ void __launch_bounds__(BWD_THREADS, K >= 2 ? 3 : 4)
 backward_kernel(DevGeom g, const float *__restrict__ proj, T *__restrict__ vol, Epilogue epi, int a_begin, int a_end,
                 const float *acc_in, float *acc_out) {
-    __shared__ double red[BWD_THREADS / 32];
     if (epi.stop && *epi.stop) return;
     auto partial_at = [&]() -> double * {
         const size_t b = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
         return epi.partial ? epi.partial + b * TILE_PARTIALS : nullptr;
     };
     if (PASSES)
-        backward_tile<T, ZFAST, CX, K, HOIST>(g, proj, vol, epi, blockIdx.x, blockIdx.y, blockIdx.z, a_begin, a_end,
-                                              acc_in, acc_out, partial_at, red);
+        backward_tile<T, ZFAST, CX, K>(g, proj, vol, epi, blockIdx.x, blockIdx.y, blockIdx.z, a_begin, a_end, acc_in,
+                                       acc_out, partial_at);
     else
-        backward_tile<T, ZFAST, CX, K, HOIST>(g, proj, vol, epi, blockIdx.x, blockIdx.y, blockIdx.z, 0, g.nangles,
-                                              nullptr, nullptr, partial_at, red);
+        backward_tile<T, ZFAST, CX, K>(g, proj, vol, epi, blockIdx.x, blockIdx.y, blockIdx.z, 0, g.nangles, nullptr,
+                                       nullptr, partial_at);
+}
+
+// Patch tiles: 2 patches of 2 x 2 columns, ZG stacks of 64 voxels.
+template <typename T, bool ZFAST, bool ALONG_X, int ZG, bool PASSES>
+__global__ void __launch_bounds__(64 * ZG, 12 / ZG)
+patch_kernel(DevGeom g, const float *__restrict__ proj, T *__restrict__ vol, Epilogue epi, int a_begin, int a_end,
+             const float *acc_in, float *acc_out) {
+    extern __shared__ float4 patch_lists[];
+    if (epi.stop && *epi.stop) return;
+    auto partial_at = [&]() -> double * {
+        const size_t b = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+        return epi.partial ? epi.partial + b * TILE_PARTIALS : nullptr;
+    };
+    if (PASSES)
+        patch_tile<T, ZFAST, 2, ALONG_X, ZG>(g, proj, vol, epi, blockIdx.x, blockIdx.y, blockIdx.z, a_begin, a_end,
+                                             acc_in, acc_out, partial_at, (char *)patch_lists);
+    else
+        patch_tile<T, ZFAST, 2, ALONG_X, ZG>(g, proj, vol, epi, blockIdx.x, blockIdx.y, blockIdx.z, 0, g.nangles,
+                                             nullptr, nullptr, partial_at, (char *)patch_lists);
 }
 
 template <typename T, bool ZF, bool PASSES>
@@ -40,20 +58,28 @@ void launch_backward_tp(const DevGeom &g, const float *y, void *x, const Epilogu
                         int a1, const float *acc_in, float *acc_out) {
     const dim3 grid = backward_grid(g);
     T *xx = (T *)x;
-#define CBCT_BWD(CX, K, HOIST)                                                                                  \
-    backward_kernel<T, ZF, CX, K, HOIST, PASSES><<<grid, BWD_THREADS, 0, s>>>(g, y, xx, epi, a0, a1, acc_in, \
-                                                                               acc_out)
+    if (backward_patches(g)) {
+        const int lists = 2 * patch_list_bytes(g.patch_columns);
+#define CBCT_PATCH(ALONG_X, ZG)                                                                                 \
+    patch_kernel<T, ZF, ALONG_X, ZG, PASSES><<<grid, 64 * ZG, lists, s>>>(g, y, xx, epi, a0, a1, acc_in, acc_out)
+        switch (g.bwd_config) {
+        case 4: CBCT_PATCH(true, 2); break;
+        case 5: CBCT_PATCH(false, 2); break;
+        case 6: CBCT_PATCH(true, 4); break;
+        default: CBCT_PATCH(false, 4); break;
+        }
+#undef CBCT_PATCH
+        return;
+    }
+#define CBCT_BWD(CX, K) \
+    backward_kernel<T, ZF, CX, K, PASSES><<<grid, BWD_THREADS, 0, s>>>(g, y, xx, epi, a0, a1, acc_in, acc_out)
     switch (g.bwd_config) {         // shapes as in backward_shape
-    case 1: CBCT_BWD(4, 2, true); break;
-    case 2: CBCT_BWD(8, 1, true); break;
-    case 3: CBCT_BWD(2, 2, true); break;
-    case 4: CBCT_BWD(4, 4, false); break;
-    case 5: CBCT_BWD(2, 4, false); break;
-    case 6: CBCT_BWD(4, 8, false); break;
-    case 7: CBCT_BWD(2, 8, false); break;
-    case 8: CBCT_BWD(2, 4, true); break;
-    case 9: CBCT_BWD(4, 4, true); break;
-    default: CBCT_BWD(4, 1, true); break;
+    case 1: CBCT_BWD(4, 2); break;
+    case 2: CBCT_BWD(8, 1); break;
+    case 3: CBCT_BWD(2, 2); break;
+    case 4: case 6: case 9: CBCT_BWD(4, 4); break;
+    case 5: case 7: case 8: CBCT_BWD(2, 4); break;
+    default: CBCT_BWD(4, 1); break;
     }
 #undef CBCT_BWD
 }
