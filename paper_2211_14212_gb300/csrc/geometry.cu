@@ -137,7 +137,7 @@ static void set_patch_bounds(DevGeom &g, const cbct_geometry_desc &d) {
     // half integers of 12 bits times 11 bits are exact (patch_crossing); a
     // slab covers more than the margins of its planes; 32-bit offsets within
     // a projection; the lists fit 48 KB of shared memory
-    if (columns > 22.0 || passed + 2.0 * 0.05 > 1.95 || rho * far < 0.25 || d.nz > 4096 || d.nv > 4096 || d.nv < 3 ||
+    if (columns > 22.0 || passed + 2.0 * 0.05 > 2.95 || rho * far < 0.25 || d.nz > 4096 || d.nv > 4096 || d.nv < 3 ||
         (int64_t)d.nu * d.nv >= (int64_t)1 << 30)
         return;
     g.patch_columns = std::max(4, (int)columns);

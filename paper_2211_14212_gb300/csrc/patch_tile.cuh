@@ -31,10 +31,12 @@
 
 namespace cbct {
 
+
 constexpr int PT_ANGLES = 8;             // angles per list
 constexpr int PT_STEP = 8;               // detector columns listed in one step of a warp (x 4 cells)
 constexpr int PT_MAX_COLUMNS = 24;       // most detector columns across a patch
 constexpr float PT_MARGIN = 0.05f;       // pixels; covers the windows' rounding (about 1e-4)
+constexpr int PT_CROSSING = 3;           // most rows that a plane passes between a patch's near and far depth
 constexpr float PT_NEVER = -FLT_MAX;     // crossing alpha of a row that enters its slab before the patch
 
 // Columns of one angle: mask[s] bit 4 c + q: detector column 8 s + c crosses
@@ -50,6 +52,11 @@ __host__ __device__ __forceinline__ int patch_list_bytes(int columns) {
     return 2 * PT_ANGLES * ((int)sizeof(PatchHead) + columns * 4 * (int)sizeof(float4));
 }
 
+__device__ __forceinline__ float fast_rcp(float v) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
 __device__ __forceinline__ float fma_sat(float a, float b, float c) { return __saturatef(__fmaf_rn(a, b, c)); }
 
 // First row above plane p (p: planes from the mid-plane, in voxels) at
@@ -70,7 +77,7 @@ __device__ __forceinline__ float patch_row(float rows, float mag, float offset) 
 // the difference is rounded at its own size only.
 __device__ __forceinline__ float patch_crossing(const DevGeom &g, float c, float p, float p_lo) {
     const float n = __fmaf_rn(p, g.rho_hi, -(c * g.m_hi)) + __fmaf_rn(-c, g.m_lo, p_lo);
-    return __fdividef(n, c);
+    return n * fast_rcp(c);
 }
 
 // Lists of one angle for the patch at (i0, j0), built by one warp, and the
@@ -87,23 +94,22 @@ __device__ __forceinline__ void patch_list(const DevGeom &g, const float *__rest
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
         const float px = (c & 1) ? x1 : x0, py = (c & 2) ? y1 : y0;
-        const float mag = __fdividef(g.dsd, g.dso - (px * cs.x + py * cs.y));
+        const float mag = g.dsd * fast_rcp(g.dso - (px * cs.x + py * cs.y));
         const float u = (py * cs.x - px * cs.y) * mag;
         umin = fminf(umin, u);
         umax = fmaxf(umax, u);
         magmin = fminf(magmin, mag);
         magmax = fmaxf(magmax, mag);
     }
-    const float inv_du = 1.0f / g.du, cu = 0.5f * (g.nu - 1), cv = 0.5f * (g.nv - 1);
+    const float inv_du = fast_rcp(g.du), cu = 0.5f * (g.nu - 1), cv = 0.5f * (g.nv - 1);
     const int iu0 = max(0, (int)ceilf(__fmaf_rn(umin, inv_du, cu - PT_MARGIN)));
     const int iu1 = min(min(g.nu - 1, iu0 + g.patch_columns - 1), (int)floorf(__fmaf_rn(umax, inv_du, cu + PT_MARGIN)));
     const int cell = lane & 3, i = i0 + (cell & 1), j = j0 + (cell >> 1);
     const bool in_volume = i < g.nx && j < g.ny;
     const float dmag = magmax - magmin;
-    unsigned mask[PT_MAX_COLUMNS / PT_STEP];
-#pragma unroll
+#pragma unroll 1
     for (int s = 0; s < PT_MAX_COLUMNS / PT_STEP; ++s) {
-        mask[s] = 0;
+        if (lane == 0) head->mask[s] = 0;
         if (iu0 + s * PT_STEP > iu1) continue;              // uniform
         const int c = s * PT_STEP + (lane >> 2), iu = iu0 + c;
         float ain = -FLT_MAX, aout = FLT_MAX;
@@ -115,9 +121,10 @@ __device__ __forceinline__ void patch_list(const DevGeom &g, const float *__rest
             clip_slab(RayAxis{xy.z, xy.w, q.y}, g.dy, j, j + 1, ain, aout, miss);
         }
         const bool crosses = !miss && ain < aout;
-        mask[s] = __ballot_sync(0xffffffffu, crosses);
+        const unsigned crossed = __ballot_sync(0xffffffffu, crosses);
+        if (lane == 0) head->mask[s] = crossed;
         if (crosses) {
-            const float len = aout - ain, inv = 1.0f / len, start = -ain * inv;
+            const float len = aout - ain, inv = fast_rcp(len), start = -ain * inv;
             entries[c * 4 + cell] = make_float4(len, len, inv, start);
             const float *wcol = wproj + ((size_t)a * g.nu + iu) * g.nv;
 #pragma unroll
@@ -128,7 +135,7 @@ __device__ __forceinline__ void patch_list(const DevGeom &g, const float *__rest
                 const int first = __float_as_int(patch_row(rows, magmin, patch_row_offset(p, cv))) - ZMAGIC_BITS;
                 const int step = p > 0.0f ? 1 : -1;
                 int row = p > 0.0f ? first : first - 1;
-                const int n = fabsf(rows) * dmag + 2.0f * PT_MARGIN > 1.0f ? 2 : 1;
+                const int n = (int)ceilf(__fmaf_rn(fabsf(rows), dmag, 2.0f * PT_MARGIN));
                 for (int t = 0; t < n; ++t, row += step) {
                     if ((unsigned)row >= (unsigned)g.nv) continue;
                     const float at = patch_crossing(g, (float)row - cv, p, p * g.rho_lo);
@@ -138,18 +145,16 @@ __device__ __forceinline__ void patch_list(const DevGeom &g, const float *__rest
         }
     }
     if (lane == 0) {
-        head->mask[0] = mask[0];
-        head->mask[1] = mask[1];
-        head->mask[2] = mask[2];
         head->base = (unsigned)iu0 * (unsigned)g.nv * 4u;
         head->mag = magmin;
         head->dmag = dmag;
     }
 }
 
-// Adds one detector column's part to the cells it crosses (bits of `cells`).
-// S: the sum of each voxel's rows, d[t]: its t-th row, at[t]: the alpha at
-// which that row enters the voxel's slab.
+// Adds one detector column's part to the cells it crosses (bits of `cells`),
+// for the lane's two voxels.  S: the sum of each voxel's rows; d[t]: its t-th
+// row from the entry plane, at[t]: the alpha at which that row enters the
+// voxel's slab.
 template <int CAND>
 __device__ __forceinline__ void patch_cells(unsigned cells, const float4 *entries, float2 S, const float2 (&d)[CAND],
                                             const float2 (&at)[CAND], float2 (&sum)[4], float2 (&before)[4]) {
@@ -168,6 +173,8 @@ __device__ __forceinline__ void patch_cells(unsigned cells, const float4 *entrie
     }
 }
 
+__device__ __forceinline__ float &half(float2 &v, int s) { return s ? v.y : v.x; }
+
 // PATCHES patches of 2 x 2 columns side by side (along x if ALONG_X, else
 // along y) and ZG stacks of 64 voxels: a tile of PATCHES * ZG warps.
 // Angles [a_begin, a_end), running sums and epilogue as in backward_tile.
@@ -176,12 +183,12 @@ template <typename T, bool ZFAST, int PATCHES, bool ALONG_X, int ZG, typename Pa
 __device__ __forceinline__ void patch_tile(const DevGeom &g, const float *__restrict__ wproj, T *__restrict__ vol,
                                            const Epilogue &epi, int tx, int ty, int tz, int a_begin, int a_end,
                                            const float *acc_in, float *acc_out, PartialAt &&partial_at, char *lists) {
-    constexpr int COLS = PATCHES * 2, SLOTS = 64 * ZG;
+    constexpr int COLS = PATCHES * 2, DEPTH = 64, SLOTS = DEPTH * ZG;
     const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
     const int patch = warp / ZG, zg = warp % ZG;
     const int i0 = tx * (ALONG_X ? COLS : 2) + (ALONG_X ? 2 * patch : 0);
     const int j0 = ty * (ALONG_X ? 2 : COLS) + (ALONG_X ? 0 : 2 * patch);
-    const int kb = tz * SLOTS, k0 = kb + zg * 64;
+    const int kb = tz * SLOTS, k0 = kb + zg * DEPTH;
     const int kend = min(kb + SLOTS, g.nz);
     const float cv = 0.5f * (g.nv - 1), mid = 0.5f * g.nz;
     auto group_sync = [&]() {
@@ -199,25 +206,12 @@ __device__ __forceinline__ void patch_tile(const DevGeom &g, const float *__rest
     const float p_edge[2] = {fminf((float)kb - mid, 0.0f), fmaxf((float)kend - mid, 0.0f)};
     float edge[2] = {0.0f, 0.0f};
 
-    // the lane's two voxels
-    float zl[2], zu[2], cl[2], cup[2], pp[2], pl[2];
-    bool down[2], live[2], middle[2];
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-        const int k = k0 + s * 32 + lane;
-        live[s] = k < g.nz;
-        const float p = (float)k - mid;
-        zl[s] = p * g.rho;
-        zu[s] = (p + 1.0f) * g.rho;
-        cl[s] = patch_row_offset(p, cv);
-        cup[s] = patch_row_offset(p + 1.0f, cv);
-        down[s] = p + 0.5f < 0.0f;
-        middle[s] = p + 0.5f == 0.0f;
-        pp[s] = down[s] ? p + 1.0f : p;
-        pl[s] = pp[s] * g.rho_lo;
-    }
-    const float zmax = fmaxf(fabsf((float)k0 - mid), fabsf((float)(k0 + 64) - mid)) * g.rho;
+    const float pk = (float)(k0 + lane) - mid;          // lower plane of the lane's first voxel, from the mid-plane
+    // every ray of the warp goes down (-1) / up (1), or not (0: the slabs around the mid-plane)
+    const int direction = (float)(k0 + DEPTH) - mid <= 0.0f ? -1 : (float)k0 - mid >= 0.0f ? 1 : 0;
+    const float zmax = fmaxf(fabsf((float)k0 - mid), fabsf((float)(k0 + DEPTH) - mid)) * g.rho;
     const size_t nuv = (size_t)g.nu * g.nv;
+    const int segments = (g.patch_columns + PT_STEP - 1) / PT_STEP;
     const unsigned col_bytes = (unsigned)g.nv * 4u;
 
     float2 sum[4], before[4];
@@ -231,116 +225,160 @@ __device__ __forceinline__ void patch_tile(const DevGeom &g, const float *__rest
                 patch_list(g, wproj, first + t, i0, j0, heads + buf * PT_ANGLES + t,
                            entries + (size_t)(buf * PT_ANGLES + t) * entry_stride, p_edge, edge);
     };
-    auto walk = [&](int a, const PatchHead *head, const float4 *ent) {
+    // Calls column(bits of the crossed cells, entries, byte offset) for every detector column of an angle.
+    auto columns = [&](const PatchHead *head, const float4 *ent, auto &&column) {
+#pragma unroll 1
+        for (int st = 0; st < segments; ++st) {
+            unsigned mask = head->mask[st];
+            unsigned col = st * PT_STEP * col_bytes;
+            const float4 *e = ent + st * PT_STEP * 4;
+#pragma unroll 1
+            for (; mask != 0; mask >>= 4, e += 4, col += col_bytes) column(mask & 15u, e, col);
+        }
+    };
+    // Voxels of at most ROWS rows, one of which may cross the entry plane.  A
+    // voxel's rows are [fb, fe) (plus ZMAGIC); the loads cover ROWS rows from
+    // `lo`, weighted m (1: the voxel's).  DIR +-1: all rows of the warp lie on
+    // the detector and all rays go one way, so that lo = fb or fe - ROWS, and
+    // the row that may cross is the first or the last one loaded; otherwise
+    // (0) that row has weight f.  Scalar arithmetic: the packed forms take no
+    // constant operands.
+    auto short_rows = [&](const float *pa, const PatchHead *head, const float4 *ent, auto rows_c, auto dir_c) {
+        constexpr int ROWS = decltype(rows_c)::value, DIR = decltype(dir_c)::value;
         const float mag = head->mag;
-        const float *pa = wproj + (size_t)a * nuv;
-        int rb[2], re[2], r0[2];
-        float c0[2];
+        float2 m[ROWS], f[DIR == 0 ? ROWS : 1], at[1];
+        unsigned o[2];
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
-            const float fb = patch_row(zl[s], mag, cl[s]), fe = patch_row(zu[s], mag, cup[s]);
-            rb[s] = __float_as_int(fb);
-            re[s] = live[s] ? __float_as_int(fe) : rb[s];
-            r0[s] = down[s] ? re[s] - 1 : rb[s];
-            c0[s] = ((down[s] ? fe - 1.0f : fb) - ZMAGIC) - cv;
+            const float p = pk + 32.0f * s;
+            float fb = patch_row(p * g.rho, mag, DIR > 0 ? cv - PT_MARGIN : DIR < 0 ? cv + PT_MARGIN : patch_row_offset(p, cv));
+            float fe = patch_row((p + 1.0f) * g.rho, mag, DIR > 0 ? cv - PT_MARGIN : patch_row_offset(p + 1.0f, cv));
+            const bool down = DIR < 0 || (DIR == 0 && p < -0.5f);
+            const float pe = down ? p + 1.0f : p;
+            const float first = down ? fe - 1.0f : fb;
+            const float c = (first - ZMAGIC) - cv;
+            float a = patch_crossing(g, c, pe, pe * g.rho_lo);
+            float lo = down ? fe - (float)ROWS : fb;
+            if (DIR == 0) {
+                lo = fminf(fmaxf(lo, ZMAGIC), ZMAGIC + (float)(g.nv - ROWS));
+                if (p == -0.5f) a = PT_NEVER;               // the slab around the mid-plane: no ray enters it
+                if (k0 + s * 32 + lane >= g.nz) fe = fb;
+                fe = fminf(fe, ZMAGIC + (float)g.nv);
+                fb = fmaxf(fb, ZMAGIC);
+            }
+            half(at[0], s) = a;
+            o[s] = (unsigned)__float_as_int(lo) * 4u + (head->base - (unsigned)ZMAGIC_BITS * 4u);
+#pragma unroll
+            for (int t = 0; t < ROWS; ++t) {
+                float w;
+                if (DIR > 0)
+                    w = __saturatef((fe - fb) - (float)t);
+                else if (DIR < 0)
+                    w = __saturatef((fe - fb) - (float)(ROWS - 1 - t));
+                else {
+                    w = __saturatef((fe - lo) - (float)t) - __saturatef((fb - lo) - (float)t);
+                    half(f[t], s) = __saturatef(1.0f - fabsf((first - lo) - (float)t));
+                }
+                half(m[t], s) = w;
+            }
         }
-        auto crossing = [&](int s, int t) {            // the t-th row of voxel s
-            const int step = down[s] ? -t : t;
-            const bool ok = (unsigned)(r0[s] + step - ZMAGIC_BITS) < (unsigned)g.nv && live[s] && !middle[s];
-            const float at = patch_crossing(g, c0[s] + (float)step, pp[s], pl[s]);
-            return ok ? at : PT_NEVER;
-        };
-        const int rows = (int)ceilf(__fmaf_rn(g.rho, mag, 1e-3f));
+        columns(head, ent, [&](unsigned cells, const float4 *e, unsigned col) {
+            const float *w0 = (const float *)((const char *)pa + (size_t)(o[0] + col));
+            const float *w1 = (const float *)((const char *)pa + (size_t)(o[1] + col));
+            float2 w[ROWS];
+#pragma unroll
+            for (int t = 0; t < ROWS; ++t) w[t] = make_float2(__ldg(w0 + t), __ldg(w1 + t));
+            float2 S = __fmul2_rn(m[0], w[0]), d[1];
+#pragma unroll
+            for (int t = 1; t < ROWS; ++t) S = __ffma2_rn(m[t], w[t], S);
+            if (DIR != 0) {
+                d[0] = w[DIR > 0 ? 0 : ROWS - 1];
+            } else {
+                d[0] = __fmul2_rn(f[0], w[0]);
+#pragma unroll
+                for (int t = 1; t < ROWS; ++t) d[0] = __ffma2_rn(f[DIR == 0 ? t : 0], w[t], d[0]);
+            }
+            patch_cells<1>(cells, e, S, d, at, sum, before);
+        });
+    };
+    auto walk = [&](const float *pa, const PatchHead *head, const float4 *ent) {
+        const float mag = head->mag;
+        const float most = __fmaf_rn(g.rho, mag, 1e-3f);
         const bool one = zmax * head->dmag + 2.0f * PT_MARGIN <= 1.0f;
-        auto short_rows = [&](auto rows_c) {
-            constexpr int ROWS = decltype(rows_c)::value;
-            unsigned off[2];
-            float2 m[ROWS];
-            bool pick[ROWS][2];
-            const float2 at[1] = {make_float2(crossing(0, 0), crossing(1, 0))};
+        typedef std::integral_constant<int, 0> C0;
+        typedef std::integral_constant<int, 1> C1;
+        typedef std::integral_constant<int, -1> CM;
+        typedef std::integral_constant<int, 2> C2;
+        typedef std::integral_constant<int, 3> C3;
+        if (one && most <= 3.0f) {
+            if (direction == 0 || __fmaf_rn(zmax, mag, 5.0f) > cv)
+                short_rows(pa, head, ent, C3(), C0());
+            else if (direction > 0)
+                most <= 2.0f ? short_rows(pa, head, ent, C2(), C1()) : short_rows(pa, head, ent, C3(), C1());
+            else
+                most <= 2.0f ? short_rows(pa, head, ent, C2(), CM()) : short_rows(pa, head, ent, C3(), CM());
+            return;
+        }
+        // any number of rows; up to PT_CROSSING of them may cross the plane
+        const int crossing_rows = (int)ceilf(__fmaf_rn(zmax, head->dmag, 2.0f * PT_MARGIN));
+        const int rows = (int)ceilf(most);
+        float2 at[PT_CROSSING];
+        int lo[2], hi[2], first[2];
 #pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                const int lo = min(max(down[s] ? re[s] - ROWS : rb[s], ZMAGIC_BITS), ZMAGIC_BITS + g.nv - ROWS);
-                off[s] = (unsigned)(lo - ZMAGIC_BITS) * 4u + head->base;
+        for (int s = 0; s < 2; ++s) {
+            const float p = pk + 32.0f * s;
+            const float fb = patch_row(p * g.rho, mag, patch_row_offset(p, cv));
+            const float fe = patch_row((p + 1.0f) * g.rho, mag, patch_row_offset(p + 1.0f, cv));
+            const bool down = p < -0.5f, live = k0 + s * 32 + lane < g.nz;
+            const float pe = down ? p + 1.0f : p;
+            const float c = ((down ? fe - 1.0f : fb) - ZMAGIC) - cv;
+            const int rb = __float_as_int(fb) - ZMAGIC_BITS, re = __float_as_int(fe) - ZMAGIC_BITS;
+            lo[s] = max(rb, 0);
+            hi[s] = live ? min(re, g.nv) : lo[s];
+            first[s] = down ? re - 1 : rb;
 #pragma unroll
-                for (int t = 0; t < ROWS; ++t) {
-                    const float f = lo + t >= rb[s] && lo + t < re[s] ? 1.0f : 0.0f;
-                    if (s == 0) m[t].x = f; else m[t].y = f;
-                    pick[t][s] = r0[s] == lo + t;
-                }
-            }
-#pragma unroll
-            for (int st = 0; st < PT_MAX_COLUMNS / PT_STEP; ++st) {
-                unsigned mask = head->mask[st];
-                const float4 *e = ent + st * PT_STEP * 4;
-                unsigned o0 = off[0] + st * PT_STEP * col_bytes, o1 = off[1] + st * PT_STEP * col_bytes;
-#pragma unroll 2
-                for (; mask != 0; mask >>= 4, e += 4, o0 += col_bytes, o1 += col_bytes) {
-                    const float *w0 = (const float *)((const char *)pa + (size_t)o0);
-                    const float *w1 = (const float *)((const char *)pa + (size_t)o1);
-                    float2 w[ROWS];
-#pragma unroll
-                    for (int t = 0; t < ROWS; ++t) w[t] = make_float2(__ldg(w0 + t), __ldg(w1 + t));
-                    float2 S = __fmul2_rn(m[0], w[0]);
-                    float2 d[1] = {w[0]};
-#pragma unroll
-                    for (int t = 1; t < ROWS; ++t) {
-                        S = __ffma2_rn(m[t], w[t], S);
-                        d[0].x = pick[t][0] ? w[t].x : d[0].x;
-                        d[0].y = pick[t][1] ? w[t].y : d[0].y;
-                    }
-                    patch_cells<1>(mask & 15u, e, S, d, at, sum, before);
-                }
-            }
-        };
-        if (one && rows <= 2) {
-            short_rows(std::integral_constant<int, 2>());
-        } else if (one && rows <= 3) {
-            short_rows(std::integral_constant<int, 3>());
-        } else {
-            // any number of rows; the first two may cross the plane
-            const float2 at[2] = {make_float2(crossing(0, 0), crossing(1, 0)),
-                                  make_float2(crossing(0, 1), crossing(1, 1))};
-            int lo[2], hi[2], dr[2][2];
-#pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                lo[s] = max(rb[s] - ZMAGIC_BITS, 0);
-                hi[s] = min(re[s] - ZMAGIC_BITS, g.nv);
-#pragma unroll
-                for (int t = 0; t < 2; ++t)
-                    dr[t][s] = min(max(r0[s] - ZMAGIC_BITS + (down[s] ? -t : t), 0), g.nv - 1);
-            }
-#pragma unroll 1
-            for (int st = 0; st < PT_MAX_COLUMNS / PT_STEP; ++st) {
-                unsigned mask = head->mask[st];
-                const float4 *e = ent + st * PT_STEP * 4;
-                const float *w = (const float *)((const char *)pa + (size_t)(head->base + st * PT_STEP * col_bytes));
-#pragma unroll 1
-                for (; mask != 0; mask >>= 4, e += 4, w += g.nv) {
-                    const float2 d[2] = {make_float2(__ldg(w + dr[0][0]), __ldg(w + dr[0][1])),
-                                         make_float2(__ldg(w + dr[1][0]), __ldg(w + dr[1][1]))};
-                    float2 S = make_float2(0.0f, 0.0f);
-#pragma unroll 4
-                    for (int t = 0; t < rows; ++t) {
-                        if (lo[0] + t < hi[0]) S.x += __ldg(w + lo[0] + t);
-                        if (lo[1] + t < hi[1]) S.y += __ldg(w + lo[1] + t);
-                    }
-                    patch_cells<2>(mask & 15u, e, S, d, at, sum, before);
-                }
+            for (int t = 0; t < PT_CROSSING; ++t) {
+                const int step = down ? -t : t;
+                const bool ok = t < crossing_rows && live && p != -0.5f && (unsigned)(first[s] + step) < (unsigned)g.nv;
+                half(at[t], s) = ok ? patch_crossing(g, c + (float)step, pe, pe * g.rho_lo) : PT_NEVER;
             }
         }
+        columns(head, ent, [&](unsigned cells, const float4 *e, unsigned col) {
+            const float *w = (const float *)((const char *)pa + (size_t)(head->base + col));
+            float2 S, d[PT_CROSSING];
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                float sum_rows = 0.0f;
+#pragma unroll 4
+                for (int t = 0; t < rows; ++t)
+                    if (lo[s] + t < hi[s]) sum_rows += __ldg(w + lo[s] + t);
+                half(S, s) = sum_rows;
+                const int step = pk + 32.0f * s < -0.5f ? -1 : 1;
+#pragma unroll
+                for (int t = 0; t < PT_CROSSING; ++t)
+                    half(d[t], s) = t < crossing_rows ? __ldg(w + min(max(first[s] + t * step, 0), g.nv - 1)) : 0.0f;
+            }
+            if (crossing_rows <= 1) {
+                const float2 d1[1] = {d[0]}, at1[1] = {at[0]};
+                patch_cells<1>(cells, e, S, d1, at1, sum, before);
+            } else {
+                patch_cells<PT_CROSSING>(cells, e, S, d, at, sum, before);
+            }
+        });
     };
 
     build(a_begin, 0);
     group_sync();
     int buf = 0;
+    const float *pa = wproj + (size_t)a_begin * nuv;
 #pragma unroll 1
     for (int a = a_begin; a < a_end; a += PT_ANGLES, buf ^= 1) {
         if (a + PT_ANGLES < a_end) build(a + PT_ANGLES, buf ^ 1);
         const int n = min(PT_ANGLES, a_end - a);
+        const PatchHead *head = heads + buf * PT_ANGLES;
+        const float4 *ent = entries + (size_t)(buf * PT_ANGLES) * entry_stride;
 #pragma unroll 1
-        for (int t = 0; t < n; ++t)
-            walk(a + t, heads + buf * PT_ANGLES + t, entries + (size_t)(buf * PT_ANGLES + t) * entry_stride);
+        for (int t = 0; t < n; ++t, ++head, ent += entry_stride, pa += nuv) walk(pa, head, ent);
         group_sync();
     }
 
@@ -350,8 +388,10 @@ __device__ __forceinline__ void patch_tile(const DevGeom &g, const float *__rest
     float *const esh = dsh + 4 * (SLOTS + 2);               // [ZG][8]
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        if (live[0]) dsh[q * (SLOTS + 2) + 1 + zg * 64 + lane] = before[q].x;
-        if (live[1]) dsh[q * (SLOTS + 2) + 33 + zg * 64 + lane] = before[q].y;
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+            if (k0 + s * 32 + lane < g.nz)
+                dsh[q * (SLOTS + 2) + 1 + zg * DEPTH + s * 32 + lane] = half(before[q], s);
     }
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
@@ -373,9 +413,9 @@ __device__ __forceinline__ void patch_tile(const DevGeom &g, const float *__rest
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
             const int k = k0 + s * 32 + lane;
-            if (!live[s] || i >= g.nx || j >= g.ny) continue;
+            if (k >= g.nz || i >= g.nx || j >= g.ny) continue;
             const float *dk = dsh + q * (SLOTS + 2) + 1 + (k - kb);
-            float v = (s == 0 ? sum[q].x : sum[q].y) - dk[0];
+            float v = half(sum[q], s) - dk[0];
             if (2 * k - 1 < g.nz) v += dk[-1];              // slab k - 1 lies below the mid-plane
             if (2 * k + 3 > g.nz) v += dk[1];
             const size_t flat = ((size_t)j * g.nx + i) * g.nz + k;
