@@ -242,8 +242,8 @@ extern "C" cbct_status cbct_geometry_create(const cbct_geometry_desc *d, cbct_ge
         dg.zsingle = zrise < 0.98 * d->dz ? 1 : 0;
     }
     set_patch_bounds(dg, *d);
-    if (dg.patch_columns > 0 && nz > 64)
-        dg.bwd_config = nz > 128 ? 7 : 5;   // patch tiles of 256 / 128 voxels along z
+    if (dg.patch_columns > 0)
+        dg.bwd_config = nz > 128 ? 7 : nz > 64 ? 5 : 3;   // patch tiles of 256 / 128 / 64 voxels along z
     else
         dg.bwd_config = nz >= 64 ? 3 : 0;   // 2 / 1 voxels per lane by column depth
     dg.angle_block = default_angle_block(dg);

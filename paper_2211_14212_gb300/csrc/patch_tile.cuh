@@ -32,7 +32,8 @@
 namespace cbct {
 
 
-constexpr int PT_ANGLES = 8;             // angles per list
+constexpr int PT_PATCHES = 2;            // patches of a tile
+constexpr int PT_ANGLES = 8;             // angles listed at a time, by all splits of a patch together
 constexpr int PT_STEP = 8;               // detector columns listed in one step of a warp (x 4 cells)
 constexpr int PT_MAX_COLUMNS = 24;       // most detector columns across a patch
 constexpr float PT_MARGIN = 0.05f;       // pixels; covers the windows' rounding (about 1e-4)
@@ -47,9 +48,18 @@ struct PatchHead {
     float mag, dmag, pad[2];
 };
 
-// bytes of one patch's two list buffers (columns: DevGeom::patch_columns)
-__host__ __device__ __forceinline__ int patch_list_bytes(int columns) {
-    return 2 * PT_ANGLES * ((int)sizeof(PatchHead) + columns * 4 * (int)sizeof(float4));
+// Bytes of a list of `angles` angles, two buffers (columns: DevGeom::patch_columns).
+__host__ __device__ __forceinline__ int patch_list_bytes(int columns, int angles) {
+    return 2 * angles * ((int)sizeof(PatchHead) + columns * 4 * (int)sizeof(float4));
+}
+
+// Shared memory of a tile of ZG stacks and SPLITS angle ranges: the lists, and
+// after the last angle the crossing parts, the edges' sums and the splits' sums.
+template <int ZG, int SPLITS>
+__host__ __device__ __forceinline__ int patch_shared_bytes(int columns) {
+    const int lists = PT_PATCHES * SPLITS * patch_list_bytes(columns, PT_ANGLES / SPLITS);
+    const int last = (int)sizeof(float) * PT_PATCHES * (4 * (64 * ZG + 2) + 8 * ZG * SPLITS + (SPLITS - 1) * ZG * 16 * 32);
+    return lists > last ? lists : last;
 }
 
 __device__ __forceinline__ float fast_rcp(float v) {
@@ -175,32 +185,38 @@ __device__ __forceinline__ void patch_cells(unsigned cells, const float4 *entrie
 
 __device__ __forceinline__ float &half(float2 &v, int s) { return s ? v.y : v.x; }
 
-// PATCHES patches of 2 x 2 columns side by side (along x if ALONG_X, else
-// along y) and ZG stacks of 64 voxels: a tile of PATCHES * ZG warps.
+// A tile: two patches of 2 x 2 columns side by side (along x if ALONG_X, else
+// along y), ZG stacks of 64 voxels, and the angles in SPLITS ranges, 8 warps
+// in all.  The splits' sums are added in order at the end; they keep the warps
+// of a volume that is not deep busy (32^3 voxels are 256 patches).
 // Angles [a_begin, a_end), running sums and epilogue as in backward_tile.
-// lists: PATCHES * patch_list_bytes(g.patch_columns) bytes of shared memory.
-template <typename T, bool ZFAST, int PATCHES, bool ALONG_X, int ZG, typename PartialAt>
+// lists: patch_shared_bytes<ZG, SPLITS>() of shared memory.
+template <typename T, bool ZFAST, bool ALONG_X, int ZG, int SPLITS, typename PartialAt>
 __device__ __forceinline__ void patch_tile(const DevGeom &g, const float *__restrict__ wproj, T *__restrict__ vol,
                                            const Epilogue &epi, int tx, int ty, int tz, int a_begin, int a_end,
                                            const float *acc_in, float *acc_out, PartialAt &&partial_at, char *lists) {
-    constexpr int COLS = PATCHES * 2, DEPTH = 64, SLOTS = DEPTH * ZG;
+    static_assert(PT_PATCHES * ZG * SPLITS == TILE_PARTIALS, "one norm partial per warp");
+    constexpr int DEPTH = 64, SLOTS = DEPTH * ZG, ANGLES = PT_ANGLES / SPLITS;
     const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
-    const int patch = warp / ZG, zg = warp % ZG;
-    const int i0 = tx * (ALONG_X ? COLS : 2) + (ALONG_X ? 2 * patch : 0);
-    const int j0 = ty * (ALONG_X ? 2 : COLS) + (ALONG_X ? 0 : 2 * patch);
+    const int zg = warp % ZG, patch = warp / ZG % PT_PATCHES, split = warp / (ZG * PT_PATCHES);
+    const int i0 = tx * (ALONG_X ? 2 * PT_PATCHES : 2) + (ALONG_X ? 2 * patch : 0);
+    const int j0 = ty * (ALONG_X ? 2 : 2 * PT_PATCHES) + (ALONG_X ? 0 : 2 * patch);
     const int kb = tz * SLOTS, k0 = kb + zg * DEPTH;
     const int kend = min(kb + SLOTS, g.nz);
+    const int angles = a_end - a_begin, group = split * PT_PATCHES + patch;
+    const int a_first = a_begin + (int)((long long)angles * split / SPLITS);
+    const int a_last = a_begin + (int)((long long)angles * (split + 1) / SPLITS);
     const float cv = 0.5f * (g.nv - 1), mid = 0.5f * g.nz;
-    auto group_sync = [&]() {
+    auto group_sync = [&]() {               // the warps that share a list
         if (ZG == 1)
             __syncwarp();
         else
-            asm volatile("bar.sync %0, %1;" ::"r"(1 + patch), "n"(32 * ZG) : "memory");
+            asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(32 * ZG) : "memory");
     };
-    char *const mine = lists + patch * patch_list_bytes(g.patch_columns);
+    char *const mine = lists + group * patch_list_bytes(g.patch_columns, ANGLES);
     const int entry_stride = g.patch_columns * 4;
     PatchHead *const heads = (PatchHead *)mine;
-    float4 *const entries = (float4 *)(mine + 2 * PT_ANGLES * sizeof(PatchHead));
+    float4 *const entries = (float4 *)(mine + 2 * ANGLES * sizeof(PatchHead));
 
     // planes at the ends of the tile's slabs, when rays cross them outwards
     const float p_edge[2] = {fminf((float)kb - mid, 0.0f), fmaxf((float)kend - mid, 0.0f)};
@@ -220,10 +236,10 @@ __device__ __forceinline__ void patch_tile(const DevGeom &g, const float *__rest
 
     auto build = [&](int first, int buf) {
 #pragma unroll 1
-        for (int t = zg; t < PT_ANGLES; t += ZG)
-            if (first + t < a_end)
-                patch_list(g, wproj, first + t, i0, j0, heads + buf * PT_ANGLES + t,
-                           entries + (size_t)(buf * PT_ANGLES + t) * entry_stride, p_edge, edge);
+        for (int t = zg; t < ANGLES; t += ZG)
+            if (first + t < a_last)
+                patch_list(g, wproj, first + t, i0, j0, heads + buf * ANGLES + t,
+                           entries + (size_t)(buf * ANGLES + t) * entry_stride, p_edge, edge);
     };
     // Calls column(bits of the crossed cells, entries, byte offset) for every detector column of an angle.
     auto columns = [&](const PatchHead *head, const float4 *ent, auto &&column) {
@@ -343,20 +359,35 @@ __device__ __forceinline__ void patch_tile(const DevGeom &g, const float *__rest
                 half(at[t], s) = ok ? patch_crossing(g, c + (float)step, pe, pe * g.rho_lo) : PT_NEVER;
             }
         }
+        // on the detector and all one way: every voxel has the first `full`
+        // rows, and the rows that may cross need no clamp
+        const bool inside = direction != 0 && __fmaf_rn(zmax, mag, most + (float)(PT_CROSSING + 2)) <= cv;
+        const int full = inside ? (int)(most - (PT_MARGIN + 2e-3f)) : 0;
+        const unsigned base = head->base;
         columns(head, ent, [&](unsigned cells, const float4 *e, unsigned col) {
-            const float *w = (const float *)((const char *)pa + (size_t)(head->base + col));
-            float2 S, d[PT_CROSSING];
+            const float *w = (const float *)((const char *)pa + (size_t)(base + col));
+            float2 S = make_float2(0.0f, 0.0f), d[PT_CROSSING];
+            const float *w0 = w + lo[0], *w1 = w + lo[1];
+#pragma unroll 2
+            for (int t = 0; t < full; ++t) S = __fadd2_rn(S, make_float2(__ldg(w0 + t), __ldg(w1 + t)));
+#pragma unroll 1
+            for (int t = full; t < rows; ++t) {
+                if (lo[0] + t < hi[0]) S.x += __ldg(w0 + t);
+                if (lo[1] + t < hi[1]) S.y += __ldg(w1 + t);
+            }
+            if (inside) {
+                const float *f0 = w + first[0], *f1 = w + first[1];
 #pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                float sum_rows = 0.0f;
-#pragma unroll 4
-                for (int t = 0; t < rows; ++t)
-                    if (lo[s] + t < hi[s]) sum_rows += __ldg(w + lo[s] + t);
-                half(S, s) = sum_rows;
-                const int step = pk + 32.0f * s < -0.5f ? -1 : 1;
+                for (int t = 0; t < PT_CROSSING; ++t, f0 += direction, f1 += direction)
+                    d[t] = t < crossing_rows ? make_float2(__ldg(f0), __ldg(f1)) : make_float2(0.0f, 0.0f);
+            } else {
 #pragma unroll
-                for (int t = 0; t < PT_CROSSING; ++t)
-                    half(d[t], s) = t < crossing_rows ? __ldg(w + min(max(first[s] + t * step, 0), g.nv - 1)) : 0.0f;
+                for (int s = 0; s < 2; ++s) {
+                    const int step = pk + 32.0f * s < -0.5f ? -1 : 1;
+#pragma unroll
+                    for (int t = 0; t < PT_CROSSING; ++t)
+                        half(d[t], s) = t < crossing_rows ? __ldg(w + min(max(first[s] + t * step, 0), g.nv - 1)) : 0.0f;
+                }
             }
             if (crossing_rows <= 1) {
                 const float2 d1[1] = {d[0]}, at1[1] = {at[0]};
@@ -367,44 +398,79 @@ __device__ __forceinline__ void patch_tile(const DevGeom &g, const float *__rest
         });
     };
 
-    build(a_begin, 0);
+    build(a_first, 0);
     group_sync();
     int buf = 0;
-    const float *pa = wproj + (size_t)a_begin * nuv;
+    const float *pa = wproj + (size_t)a_first * nuv;
 #pragma unroll 1
-    for (int a = a_begin; a < a_end; a += PT_ANGLES, buf ^= 1) {
-        if (a + PT_ANGLES < a_end) build(a + PT_ANGLES, buf ^ 1);
-        const int n = min(PT_ANGLES, a_end - a);
-        const PatchHead *head = heads + buf * PT_ANGLES;
-        const float4 *ent = entries + (size_t)(buf * PT_ANGLES) * entry_stride;
+    for (int a = a_first; a < a_last; a += ANGLES, buf ^= 1) {
+        if (a + ANGLES < a_last) build(a + ANGLES, buf ^ 1);
+        if (k0 < g.nz) {                    // a warp past the volume only helps with the lists
+            const int n = min(ANGLES, a_last - a);
+            const PatchHead *head = heads + buf * ANGLES;
+            const float4 *ent = entries + (size_t)(buf * ANGLES) * entry_stride;
 #pragma unroll 1
-        for (int t = 0; t < n; ++t, ++head, ent += entry_stride, pa += nuv) walk(pa, head, ent);
+            for (int t = 0; t < n; ++t, ++head, ent += entry_stride, pa += nuv) walk(pa, head, ent);
+        }
         group_sync();
+    }
+
+    // Add the splits' sums, in order, to the first split's.
+    float *const dsh = (float *)lists + patch * 4 * (SLOTS + 2);                        // [patch][4][SLOTS + 2]
+    float *const esh = (float *)lists + PT_PATCHES * 4 * (SLOTS + 2) + patch * 8 * ZG * SPLITS;
+    float *const rsh = (float *)lists + PT_PATCHES * (4 * (SLOTS + 2) + 8 * ZG * SPLITS);
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        for (int o = 4; o < 32; o <<= 1) edge[e] += __shfl_xor_sync(0xffffffffu, edge[e], o);
+        if (lane < 4) esh[(split * ZG + zg) * 8 + e * 4 + lane] = edge[e];
+    }
+    if (SPLITS > 1) {
+        float *const own = rsh + ((patch * ZG + zg) * 16) * 32 + lane;
+        constexpr int STRIDE = PT_PATCHES * ZG * 16 * 32;
+        if (split > 0) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                float *const to = own + (split - 1) * STRIDE + q * 4 * 32;
+                to[0] = sum[q].x;
+                to[32] = sum[q].y;
+                to[64] = before[q].x;
+                to[96] = before[q].y;
+            }
+        }
+        __syncthreads();
+        if (split == 0) {
+#pragma unroll 1
+            for (int o = 0; o < SPLITS - 1; ++o) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float *const from = own + o * STRIDE + q * 4 * 32;
+                    sum[q].x += from[0];
+                    sum[q].y += from[32];
+                    before[q].x += from[64];
+                    before[q].y += from[96];
+                }
+            }
+        }
     }
 
     // Move the crossing parts: slot k of D goes to voxel k + 1 below the
     // mid-plane and to voxel k - 1 above it; the tile's ends come from `edge`.
-    float *const dsh = (float *)mine;                       // [4][SLOTS + 2]
-    float *const esh = dsh + 4 * (SLOTS + 2);               // [ZG][8]
+    if (split == 0) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < 4; ++q) {
 #pragma unroll
-        for (int s = 0; s < 2; ++s)
-            if (k0 + s * 32 + lane < g.nz)
-                dsh[q * (SLOTS + 2) + 1 + zg * DEPTH + s * 32 + lane] = half(before[q], s);
+            for (int s = 0; s < 2; ++s)
+                if (k0 + s * 32 + lane < g.nz) dsh[q * (SLOTS + 2) + 1 + zg * DEPTH + s * 32 + lane] = half(before[q], s);
+        }
     }
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-        for (int o = 4; o < 32; o <<= 1) edge[e] += __shfl_xor_sync(0xffffffffu, edge[e], o);
-        if (lane < 4) esh[zg * 8 + e * 4 + lane] = edge[e];
+    __syncthreads();
+    if (split == 0 && zg == 0 && lane < 8) {
+        float v = 0.0f;
+        for (int w = 0; w < ZG * SPLITS; ++w) v += esh[w * 8 + lane];
+        dsh[(lane & 3) * (SLOTS + 2) + (lane < 4 ? 0 : 1 + kend - kb)] = v;
     }
-    group_sync();
-    if (zg == 0 && lane < 8) {
-        float s = 0.0f;
-        for (int z = 0; z < ZG; ++z) s += esh[z * 8 + lane];
-        dsh[(lane & 3) * (SLOTS + 2) + (lane < 4 ? 0 : 1 + kend - kb)] = s;
-    }
-    group_sync();
+    __syncthreads();
     const double acoef = epi_a(epi), bcoef = epi_b(epi);
     double sq = 0.0;
 #pragma unroll
@@ -413,7 +479,7 @@ __device__ __forceinline__ void patch_tile(const DevGeom &g, const float *__rest
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
             const int k = k0 + s * 32 + lane;
-            if (k >= g.nz || i >= g.nx || j >= g.ny) continue;
+            if (split > 0 || k >= g.nz || i >= g.nx || j >= g.ny) continue;
             const float *dk = dsh + q * (SLOTS + 2) + 1 + (k - kb);
             float v = half(sum[q], s) - dk[0];
             if (2 * k - 1 < g.nz) v += dk[-1];              // slab k - 1 lies below the mid-plane
@@ -436,11 +502,7 @@ __device__ __forceinline__ void patch_tile(const DevGeom &g, const float *__rest
         }
     }
     double *partial = acc_out ? nullptr : partial_at();
-    if (partial) {
-        warp_partial(sq, partial);
-        if (PATCHES * ZG < TILE_PARTIALS && lane == 0)
-            for (int w = PATCHES * ZG + warp; w < TILE_PARTIALS; w += PATCHES * ZG) partial[w] = 0.0;
-    }
+    if (partial) warp_partial(sq, partial);
 }
 
 }  // namespace cbct

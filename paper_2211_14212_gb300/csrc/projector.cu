@@ -125,9 +125,11 @@ cbct_status launch_count(const DevGeom &g, unsigned long long *count_dev, cudaSt
 
 // ---------------------------------------------------------- transpose A^T y
 
-// Transpose tile shapes.  4..7 are patch tiles where the geometry allows them
-// (DevGeom::patch_columns) and the 4-voxel tiles 9 and 8 elsewhere.
-bool backward_patches(const DevGeom &g) { return g.patch_columns > 0 && g.bwd_config >= 4 && g.bwd_config <= 7; }
+// Transpose tile shapes.  1 and 3..7 are patch tiles where the geometry allows
+// them (DevGeom::patch_columns); elsewhere 4..7 run as the 4-voxel tiles 9, 8.
+bool backward_patches(const DevGeom &g) {
+    return g.patch_columns > 0 && (g.bwd_config == 1 || (g.bwd_config >= 3 && g.bwd_config <= 7));
+}
 
 BrickShape backward_shape(const DevGeom &g) {
     const bool patches = backward_patches(g);

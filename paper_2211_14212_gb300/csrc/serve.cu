@@ -33,7 +33,7 @@
 #include <vector>
 
 #include "gk.cuh"
-#include "projector_device.cuh"
+#include "patch_tile.cuh"
 
 namespace cbct {
 
@@ -41,8 +41,14 @@ constexpr int SRV_MAX_SLOTS = 64;
 constexpr int SRV_FWD_ROWS = 4;                       // forward tile: 4 rays per lane
 constexpr int64_t SRV_SAT_TILES = 2048;                // forward tiles (8 columns x 128 rows) that fill a step
 constexpr int SRV_SRPT_AGE_CAP = 64;                   // SRPT: steps a slot may be passed over before it goes first
-constexpr int SRV_CX = 2, SRV_BK = 2;                  // transpose tile: 2 x 4 columns x 64 (configuration 3)
-constexpr int SRV_BWD_CONFIG = 3;
+// Transpose tiles: 2 x 4 columns x 64 (configuration 3), or patch tiles of 128
+// voxels along z (configuration 5) for volumes deeper than 64.  A scan whose
+// patches reach more than SRV_COLUMNS detector columns takes the tile that
+// needs no lists: the lists of all CTAs have the size of the largest.
+constexpr int SRV_CX = 2, SRV_BK = 2;
+constexpr int SRV_BWD_CONFIG = 3, SRV_BWD_DEEP = 5;
+constexpr int SRV_COLUMNS = 12;
+const int SRV_LISTS = std::max(patch_shared_bytes<1, 4>(SRV_COLUMNS), patch_shared_bytes<2, 2>(SRV_COLUMNS));
 
 struct SlotDev {
     DevGeom g;
@@ -119,6 +125,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) srv_forward(const SlotTable *t
 
 // V <- ba * A^T U + bb * V for every slot (transpose tiles of all slots, z-fastest volumes).
 __global__ void __launch_bounds__(BWD_THREADS, 4) srv_backward(const SlotTable *tab, unsigned *counter) {
+    extern __shared__ float4 patch_lists[];
     __shared__ int item_sh;
     __shared__ DevGeom g_sh;               // the claimed tile's geometry
     const int n = tab->n;
@@ -132,9 +139,16 @@ __global__ void __launch_bounds__(BWD_THREADS, 4) srv_backward(const SlotTable *
         const int local = item - tab->bwd_start[s];
         const int tbx = local % sd.bgx, tby = (local / sd.bgx) % sd.bgy, tbz = local / (sd.bgx * sd.bgy);
         const Epilogue epi{&sd.st->ba, &sd.st->bb, 0.0, 0.0, nullptr, nullptr, nullptr};
-        backward_tile<float, true, SRV_CX, SRV_BK, 2>(g_sh, sd.Uw, sd.V, epi, tbx, tby, tbz, 0, g_sh.nangles,
-                                                         nullptr, nullptr,
-                                                         [&]() { return sd.pb + (size_t)local * TILE_PARTIALS; });
+        auto partial_at = [&]() { return sd.pb + (size_t)local * TILE_PARTIALS; };
+        if (g_sh.patch_columns == 0)
+            backward_tile<float, true, SRV_CX, SRV_BK, 2>(g_sh, sd.Uw, sd.V, epi, tbx, tby, tbz, 0, g_sh.nangles,
+                                                          nullptr, nullptr, partial_at);
+        else if (g_sh.bwd_config == SRV_BWD_DEEP)
+            patch_tile<float, true, false, 2, 2>(g_sh, sd.Uw, sd.V, epi, tbx, tby, tbz, 0, g_sh.nangles, nullptr,
+                                                 nullptr, partial_at, (char *)patch_lists);
+        else
+            patch_tile<float, true, false, 1, 4>(g_sh, sd.Uw, sd.V, epi, tbx, tby, tbz, 0, g_sh.nangles, nullptr,
+                                                 nullptr, partial_at, (char *)patch_lists);
     }
 }
 
@@ -226,7 +240,8 @@ struct Slot {
     cudaGraphExec_t solo_graph = nullptr;   // captured step of this slot alone (enqueue_step)
 };
 
-// Forward tiles and bricks of a scan under the server's launch shapes.
+// Forward tiles and bricks of a scan under the server's launch shapes (the
+// deep transpose tiles are fewer).
 void grids(const cbct_geometry_desc &d, int &fgx, int &fgy, int &bgx, int &bgy, int &bgz) {
     fgx = (d.nu + FWD_COLS - 1) / FWD_COLS;
     fgy = (d.nv + 32 * SRV_FWD_ROWS - 1) / (32 * SRV_FWD_ROWS);
@@ -325,7 +340,8 @@ cbct_status ServerImpl::setup_slot(Slot &sl) {
     cbct_status st = cbct_geometry_create(&r.desc, &sl.geom);
     if (st != CBCT_OK) return st;
     sl.geom->dev.fwd_rows = SRV_FWD_ROWS;
-    sl.geom->dev.bwd_config = SRV_BWD_CONFIG;
+    if (sl.geom->dev.patch_columns > SRV_COLUMNS) sl.geom->dev.patch_columns = 0;
+    sl.geom->dev.bwd_config = sl.geom->dev.patch_columns > 0 && sl.geom->dev.nz > 64 ? SRV_BWD_DEEP : SRV_BWD_CONFIG;
     const DevGeom &g = sl.geom->dev;
     // m: a volume-side vector in the padded z-fastest layout (pads zeroed below)
     const int64_t n = cbct_geometry_num_rays(sl.geom), m = zf_len(g);
@@ -498,7 +514,7 @@ cbct_status ServerImpl::enqueue_step() {
             if (e0 != cudaSuccess) return e0;
             srv_forward<<<fwd_grid, FWD_THREADS, 0, s>>>(tab_dev, counters);
             srv_after_forward<<<SRV_MAX_SLOTS, RED_THREADS, 0, s>>>(tab_dev);
-            srv_backward<<<bwd_grid, BWD_THREADS, 0, s>>>(tab_dev, counters + 1);
+            srv_backward<<<bwd_grid, BWD_THREADS, SRV_LISTS, s>>>(tab_dev, counters + 1);
             srv_after_backward<<<SRV_MAX_SLOTS, RED_THREADS, 0, s>>>(tab_dev);
         }
         srv_update<<<vec_grid, VEC_THREADS, 0, s>>>(tab_dev);
@@ -818,7 +834,7 @@ extern "C" cbct_status cbct_server_create(const cbct_server_opts *o, cbct_server
     int sms = 0, occ_f = 0, occ_b = 0;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, S.device);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_f, srv_forward, FWD_THREADS, 0);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_b, srv_backward, BWD_THREADS, 0);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_b, srv_backward, BWD_THREADS, SRV_LISTS);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&S.s, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&S.s_admit, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&S.s_read, cudaStreamNonBlocking);

@@ -34,12 +34,11 @@ backward_kernel(DevGeom g, const float *__restrict__ proj, T *__restrict__ vol, 
                                        nullptr, partial_at);
 }
 
-// Patch tiles: 2 patches of 2 x 2 columns, ZG stacks of 64 voxels.  32 warps
-// per SM (64 registers): A^T y at 256^3 / 512^2 / 90 angles 2.80 ms, with 24
-// warps (80 registers) 3.07 ms; four voxels per lane take 20 % fewer
-// instructions but leave 16 warps and measured 3.13 ms.
-template <typename T, bool ZFAST, bool ALONG_X, int ZG, bool PASSES>
-__global__ void __launch_bounds__(64 * ZG, 16 / ZG)
+// Patch tiles.  32 warps per SM (64 registers): A^T y at 256^3 / 512^2 / 90
+// angles 2.80 ms, with 24 warps (80 registers) 3.07 ms; four voxels per lane
+// take 20 % fewer instructions but leave 16 warps and measured 3.13 ms.
+template <typename T, bool ZFAST, bool ALONG_X, int ZG, int SPLITS, bool PASSES>
+__global__ void __launch_bounds__(BWD_THREADS, 4)
 patch_kernel(DevGeom g, const float *__restrict__ proj, T *__restrict__ vol, Epilogue epi, int a_begin, int a_end,
              const float *acc_in, float *acc_out) {
     extern __shared__ float4 patch_lists[];
@@ -49,11 +48,11 @@ patch_kernel(DevGeom g, const float *__restrict__ proj, T *__restrict__ vol, Epi
         return epi.partial ? epi.partial + b * TILE_PARTIALS : nullptr;
     };
     if (PASSES)
-        patch_tile<T, ZFAST, 2, ALONG_X, ZG>(g, proj, vol, epi, blockIdx.x, blockIdx.y, blockIdx.z, a_begin, a_end,
-                                             acc_in, acc_out, partial_at, (char *)patch_lists);
+        patch_tile<T, ZFAST, ALONG_X, ZG, SPLITS>(g, proj, vol, epi, blockIdx.x, blockIdx.y, blockIdx.z, a_begin,
+                                                  a_end, acc_in, acc_out, partial_at, (char *)patch_lists);
     else
-        patch_tile<T, ZFAST, 2, ALONG_X, ZG>(g, proj, vol, epi, blockIdx.x, blockIdx.y, blockIdx.z, 0, g.nangles,
-                                             nullptr, nullptr, partial_at, (char *)patch_lists);
+        patch_tile<T, ZFAST, ALONG_X, ZG, SPLITS>(g, proj, vol, epi, blockIdx.x, blockIdx.y, blockIdx.z, 0, g.nangles,
+                                                  nullptr, nullptr, partial_at, (char *)patch_lists);
 }
 
 template <typename T, bool ZF, bool PASSES>
@@ -62,14 +61,17 @@ void launch_backward_tp(const DevGeom &g, const float *y, void *x, const Epilogu
     const dim3 grid = backward_grid(g);
     T *xx = (T *)x;
     if (backward_patches(g)) {
-        const int lists = 2 * patch_list_bytes(g.patch_columns);
-#define CBCT_PATCH(ALONG_X, ZG)                                                                                 \
-    patch_kernel<T, ZF, ALONG_X, ZG, PASSES><<<grid, 64 * ZG, lists, s>>>(g, y, xx, epi, a0, a1, acc_in, acc_out)
-        switch (g.bwd_config) {
-        case 4: CBCT_PATCH(true, 2); break;
-        case 5: CBCT_PATCH(false, 2); break;
-        case 6: CBCT_PATCH(true, 4); break;
-        default: CBCT_PATCH(false, 4); break;
+#define CBCT_PATCH(ALONG_X, ZG, SPLITS)                                                                       \
+    patch_kernel<T, ZF, ALONG_X, ZG, SPLITS, PASSES>                                                          \
+        <<<grid, BWD_THREADS, patch_shared_bytes<ZG, SPLITS>(g.patch_columns), s>>>(g, y, xx, epi, a0, a1, acc_in, \
+                                                                                    acc_out)
+        switch (g.bwd_config) {     // stacks of 64 voxels x angle ranges
+        case 1: CBCT_PATCH(true, 1, 4); break;
+        case 3: CBCT_PATCH(false, 1, 4); break;
+        case 4: CBCT_PATCH(true, 2, 2); break;
+        case 5: CBCT_PATCH(false, 2, 2); break;
+        case 6: CBCT_PATCH(true, 4, 1); break;
+        default: CBCT_PATCH(false, 4, 1); break;
         }
 #undef CBCT_PATCH
         return;
