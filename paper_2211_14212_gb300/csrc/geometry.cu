@@ -125,6 +125,10 @@ static void set_patch_bounds(DevGeom &g, const cbct_geometry_desc &d) {
     g.m_hi = leading(m);
     g.m_lo = (float)(m - g.m_hi);
     g.patch_columns = 0;
+    // fewer tiles of two patches than two for every SM: halve the tiles and
+    // the angles each warp walks (a single A^T y with 23 angles of 40 x 36 x 28
+    // voxels: 26.7 -> 21.4 us)
+    g.patch_single = d.nz <= 64 && (int64_t)((d.nx + 1) / 2) * ((d.ny + 3) / 4) < 304;
     // a patch may reach one voxel out of the volume
     const double r = std::hypot((0.5 * d.nx + 1.0) * d.dx, (0.5 * d.ny + 1.0) * d.dy);
     if (r >= 0.95 * d.dso) return;

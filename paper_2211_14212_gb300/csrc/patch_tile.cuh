@@ -32,7 +32,6 @@
 namespace cbct {
 
 
-constexpr int PT_PATCHES = 2;            // patches of a tile
 constexpr int PT_ANGLES = 8;             // angles listed at a time, by all splits of a patch together
 constexpr int PT_STEP = 8;               // detector columns listed in one step of a warp (x 4 cells)
 constexpr int PT_MAX_COLUMNS = 24;       // most detector columns across a patch
@@ -53,12 +52,12 @@ __host__ __device__ __forceinline__ int patch_list_bytes(int columns, int angles
     return 2 * angles * ((int)sizeof(PatchHead) + columns * 4 * (int)sizeof(float4));
 }
 
-// Shared memory of a tile of ZG stacks and SPLITS angle ranges: the lists, and
+// Shared memory of a tile of PATCHES patches, ZG stacks and SPLITS angle ranges: the lists, and
 // after the last angle the crossing parts, the edges' sums and the splits' sums.
-template <int ZG, int SPLITS>
+template <int PATCHES, int ZG, int SPLITS>
 __host__ __device__ __forceinline__ int patch_shared_bytes(int columns) {
-    const int lists = PT_PATCHES * SPLITS * patch_list_bytes(columns, PT_ANGLES / SPLITS);
-    const int last = (int)sizeof(float) * PT_PATCHES * (4 * (64 * ZG + 2) + 8 * ZG * SPLITS + (SPLITS - 1) * ZG * 16 * 32);
+    const int lists = PATCHES * SPLITS * patch_list_bytes(columns, PT_ANGLES / SPLITS);
+    const int last = (int)sizeof(float) * PATCHES * (4 * (64 * ZG + 2) + 8 * ZG * SPLITS + (SPLITS - 1) * ZG * 16 * 32);
     return lists > last ? lists : last;
 }
 
@@ -185,25 +184,25 @@ __device__ __forceinline__ void patch_cells(unsigned cells, const float4 *entrie
 
 __device__ __forceinline__ float &half(float2 &v, int s) { return s ? v.y : v.x; }
 
-// A tile: two patches of 2 x 2 columns side by side (along x if ALONG_X, else
-// along y), ZG stacks of 64 voxels, and the angles in SPLITS ranges, 8 warps
-// in all.  The splits' sums are added in order at the end; they keep the warps
-// of a volume that is not deep busy (32^3 voxels are 256 patches).
+// A tile: PATCHES patches of 2 x 2 columns side by side (along x if ALONG_X,
+// else along y), ZG stacks of 64 voxels, and the angles in SPLITS ranges, 8
+// warps in all.  The splits' sums are added in order at the end; they keep the
+// GPU busy with a volume that is not deep (32^3 voxels are 256 patches).
 // Angles [a_begin, a_end), running sums and epilogue as in backward_tile.
-// lists: patch_shared_bytes<ZG, SPLITS>() of shared memory.
-template <typename T, bool ZFAST, bool ALONG_X, int ZG, int SPLITS, typename PartialAt>
+// lists: patch_shared_bytes<PATCHES, ZG, SPLITS>() of shared memory.
+template <typename T, bool ZFAST, int PATCHES, bool ALONG_X, int ZG, int SPLITS, typename PartialAt>
 __device__ __forceinline__ void patch_tile(const DevGeom &g, const float *__restrict__ wproj, T *__restrict__ vol,
                                            const Epilogue &epi, int tx, int ty, int tz, int a_begin, int a_end,
                                            const float *acc_in, float *acc_out, PartialAt &&partial_at, char *lists) {
-    static_assert(PT_PATCHES * ZG * SPLITS == TILE_PARTIALS, "one norm partial per warp");
+    static_assert(PATCHES * ZG * SPLITS == TILE_PARTIALS, "one norm partial per warp");
     constexpr int DEPTH = 64, SLOTS = DEPTH * ZG, ANGLES = PT_ANGLES / SPLITS;
     const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
-    const int zg = warp % ZG, patch = warp / ZG % PT_PATCHES, split = warp / (ZG * PT_PATCHES);
-    const int i0 = tx * (ALONG_X ? 2 * PT_PATCHES : 2) + (ALONG_X ? 2 * patch : 0);
-    const int j0 = ty * (ALONG_X ? 2 : 2 * PT_PATCHES) + (ALONG_X ? 0 : 2 * patch);
+    const int zg = warp % ZG, patch = warp / ZG % PATCHES, split = warp / (ZG * PATCHES);
+    const int i0 = tx * (ALONG_X ? 2 * PATCHES : 2) + (ALONG_X ? 2 * patch : 0);
+    const int j0 = ty * (ALONG_X ? 2 : 2 * PATCHES) + (ALONG_X ? 0 : 2 * patch);
     const int kb = tz * SLOTS, k0 = kb + zg * DEPTH;
     const int kend = min(kb + SLOTS, g.nz);
-    const int angles = a_end - a_begin, group = split * PT_PATCHES + patch;
+    const int angles = a_end - a_begin, group = split * PATCHES + patch;
     const int a_first = a_begin + (int)((long long)angles * split / SPLITS);
     const int a_last = a_begin + (int)((long long)angles * (split + 1) / SPLITS);
     const float cv = 0.5f * (g.nv - 1), mid = 0.5f * g.nz;
@@ -417,8 +416,8 @@ __device__ __forceinline__ void patch_tile(const DevGeom &g, const float *__rest
 
     // Add the splits' sums, in order, to the first split's.
     float *const dsh = (float *)lists + patch * 4 * (SLOTS + 2);                        // [patch][4][SLOTS + 2]
-    float *const esh = (float *)lists + PT_PATCHES * 4 * (SLOTS + 2) + patch * 8 * ZG * SPLITS;
-    float *const rsh = (float *)lists + PT_PATCHES * (4 * (SLOTS + 2) + 8 * ZG * SPLITS);
+    float *const esh = (float *)lists + PATCHES * 4 * (SLOTS + 2) + patch * 8 * ZG * SPLITS;
+    float *const rsh = (float *)lists + PATCHES * (4 * (SLOTS + 2) + 8 * ZG * SPLITS);
     __syncthreads();
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
@@ -427,7 +426,7 @@ __device__ __forceinline__ void patch_tile(const DevGeom &g, const float *__rest
     }
     if (SPLITS > 1) {
         float *const own = rsh + ((patch * ZG + zg) * 16) * 32 + lane;
-        constexpr int STRIDE = PT_PATCHES * ZG * 16 * 32;
+        constexpr int STRIDE = PATCHES * ZG * 16 * 32;
         if (split > 0) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {

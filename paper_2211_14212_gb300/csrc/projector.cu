@@ -133,6 +133,7 @@ bool backward_patches(const DevGeom &g) {
 
 BrickShape backward_shape(const DevGeom &g) {
     const bool patches = backward_patches(g);
+    if (patches && g.patch_single && (g.bwd_config == 1 || g.bwd_config == 3)) return BrickShape{2, 2, 64};
     switch (g.bwd_config) {
     case 1: return BrickShape{4, 2, 64};
     case 2: return BrickShape{8, 1, 32};
@@ -218,20 +219,24 @@ cudaError_t launch_zbox(const DevGeom &g, float2 *zbox) {
 // formed once per product (here, or in the forward epilogue).
 
 // v-fastest y[a][iu][iv] -> w[a][iu][iv]: one thread per detector pixel,
-// looping over the angles (the length is loaded once).
+// looping over its block row's angles (the length is loaded once).  Small
+// detectors take more block rows: 64^2 pixels x 60 angles 10.1 us with one row
+// of 16 blocks, every thread waiting for 60 loads in turn; CGLS at that size
+// took 2.00 ms for 20 iterations so, 1.67 with these rows and the smaller
+// transpose tiles.
 template <typename T>
 __global__ void __launch_bounds__(256) weight_kernel(const T *__restrict__ y, const float *__restrict__ len,
                                                      float *__restrict__ w, size_t nuv, int nangles) {
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nuv; i += (size_t)gridDim.x * blockDim.x) {
         const float l = len[i];
-        for (int a = 0; a < nangles; ++a) w[(size_t)a * nuv + i] = l * Storage<T>::load(y + (size_t)a * nuv + i);
+        for (int a = blockIdx.y; a < nangles; a += gridDim.y) w[(size_t)a * nuv + i] = l * Storage<T>::load(y + (size_t)a * nuv + i);
     }
 }
 
 cbct_status launch_weight(const DevGeom &g, const void *y, cbct_dtype t, float *w, cudaStream_t s) {
     const size_t nuv = (size_t)g.nu * g.nv;
-    const int blocks = (int)std::min<size_t>((nuv + 255) / 256, 4096);
-    const int na = g.nangles;
+    const int na = g.nangles, columns = (int)std::min<size_t>((nuv + 255) / 256, 4096);
+    const dim3 blocks(columns, std::min(na, (1215 + columns) / columns));       // at least 8 blocks per SM
     switch (t) {
     case CBCT_F32: weight_kernel<float><<<blocks, 256, 0, s>>>((const float *)y, g.ray_len, w, nuv, na); break;
     case CBCT_F16: weight_kernel<__half><<<blocks, 256, 0, s>>>((const __half *)y, g.ray_len, w, nuv, na); break;

@@ -48,7 +48,7 @@ constexpr int SRV_SRPT_AGE_CAP = 64;                   // SRPT: steps a slot may
 constexpr int SRV_CX = 2, SRV_BK = 2;
 constexpr int SRV_BWD_CONFIG = 3, SRV_BWD_DEEP = 5;
 constexpr int SRV_COLUMNS = 12;
-const int SRV_LISTS = std::max(patch_shared_bytes<1, 4>(SRV_COLUMNS), patch_shared_bytes<2, 2>(SRV_COLUMNS));
+const int SRV_LISTS = std::max(patch_shared_bytes<2, 1, 4>(SRV_COLUMNS), patch_shared_bytes<2, 2, 2>(SRV_COLUMNS));
 
 struct SlotDev {
     DevGeom g;
@@ -144,10 +144,10 @@ __global__ void __launch_bounds__(BWD_THREADS, 4) srv_backward(const SlotTable *
             backward_tile<float, true, SRV_CX, SRV_BK, 2>(g_sh, sd.Uw, sd.V, epi, tbx, tby, tbz, 0, g_sh.nangles,
                                                           nullptr, nullptr, partial_at);
         else if (g_sh.bwd_config == SRV_BWD_DEEP)
-            patch_tile<float, true, false, 2, 2>(g_sh, sd.Uw, sd.V, epi, tbx, tby, tbz, 0, g_sh.nangles, nullptr,
+            patch_tile<float, true, 2, false, 2, 2>(g_sh, sd.Uw, sd.V, epi, tbx, tby, tbz, 0, g_sh.nangles, nullptr,
                                                  nullptr, partial_at, (char *)patch_lists);
         else
-            patch_tile<float, true, false, 1, 4>(g_sh, sd.Uw, sd.V, epi, tbx, tby, tbz, 0, g_sh.nangles, nullptr,
+            patch_tile<float, true, 2, false, 1, 4>(g_sh, sd.Uw, sd.V, epi, tbx, tby, tbz, 0, g_sh.nangles, nullptr,
                                                  nullptr, partial_at, (char *)patch_lists);
     }
 }
@@ -340,6 +340,7 @@ cbct_status ServerImpl::setup_slot(Slot &sl) {
     cbct_status st = cbct_geometry_create(&r.desc, &sl.geom);
     if (st != CBCT_OK) return st;
     sl.geom->dev.fwd_rows = SRV_FWD_ROWS;
+    sl.geom->dev.patch_single = 0;          // one tile shape per depth, as srv_backward has them
     if (sl.geom->dev.patch_columns > SRV_COLUMNS) sl.geom->dev.patch_columns = 0;
     sl.geom->dev.bwd_config = sl.geom->dev.patch_columns > 0 && sl.geom->dev.nz > 64 ? SRV_BWD_DEEP : SRV_BWD_CONFIG;
     const DevGeom &g = sl.geom->dev;

@@ -37,7 +37,7 @@ backward_kernel(DevGeom g, const float *__restrict__ proj, T *__restrict__ vol, 
 // Patch tiles.  32 warps per SM (64 registers): A^T y at 256^3 / 512^2 / 90
 // angles 2.80 ms, with 24 warps (80 registers) 3.07 ms; four voxels per lane
 // take 20 % fewer instructions but leave 16 warps and measured 3.13 ms.
-template <typename T, bool ZFAST, bool ALONG_X, int ZG, int SPLITS, bool PASSES>
+template <typename T, bool ZFAST, int PATCHES, bool ALONG_X, int ZG, int SPLITS, bool PASSES>
 __global__ void __launch_bounds__(BWD_THREADS, 4)
 patch_kernel(DevGeom g, const float *__restrict__ proj, T *__restrict__ vol, Epilogue epi, int a_begin, int a_end,
              const float *acc_in, float *acc_out) {
@@ -48,10 +48,10 @@ patch_kernel(DevGeom g, const float *__restrict__ proj, T *__restrict__ vol, Epi
         return epi.partial ? epi.partial + b * TILE_PARTIALS : nullptr;
     };
     if (PASSES)
-        patch_tile<T, ZFAST, ALONG_X, ZG, SPLITS>(g, proj, vol, epi, blockIdx.x, blockIdx.y, blockIdx.z, a_begin,
+        patch_tile<T, ZFAST, PATCHES, ALONG_X, ZG, SPLITS>(g, proj, vol, epi, blockIdx.x, blockIdx.y, blockIdx.z, a_begin,
                                                   a_end, acc_in, acc_out, partial_at, (char *)patch_lists);
     else
-        patch_tile<T, ZFAST, ALONG_X, ZG, SPLITS>(g, proj, vol, epi, blockIdx.x, blockIdx.y, blockIdx.z, 0, g.nangles,
+        patch_tile<T, ZFAST, PATCHES, ALONG_X, ZG, SPLITS>(g, proj, vol, epi, blockIdx.x, blockIdx.y, blockIdx.z, 0, g.nangles,
                                                   nullptr, nullptr, partial_at, (char *)patch_lists);
 }
 
@@ -61,17 +61,24 @@ void launch_backward_tp(const DevGeom &g, const float *y, void *x, const Epilogu
     const dim3 grid = backward_grid(g);
     T *xx = (T *)x;
     if (backward_patches(g)) {
-#define CBCT_PATCH(ALONG_X, ZG, SPLITS)                                                                       \
-    patch_kernel<T, ZF, ALONG_X, ZG, SPLITS, PASSES>                                                          \
-        <<<grid, BWD_THREADS, patch_shared_bytes<ZG, SPLITS>(g.patch_columns), s>>>(g, y, xx, epi, a0, a1, acc_in, \
-                                                                                    acc_out)
-        switch (g.bwd_config) {     // stacks of 64 voxels x angle ranges
-        case 1: CBCT_PATCH(true, 1, 4); break;
-        case 3: CBCT_PATCH(false, 1, 4); break;
-        case 4: CBCT_PATCH(true, 2, 2); break;
-        case 5: CBCT_PATCH(false, 2, 2); break;
-        case 6: CBCT_PATCH(true, 4, 1); break;
-        default: CBCT_PATCH(false, 4, 1); break;
+#define CBCT_PATCH(PATCHES, ALONG_X, ZG, SPLITS)                                                               \
+    patch_kernel<T, ZF, PATCHES, ALONG_X, ZG, SPLITS, PASSES>                                                  \
+        <<<grid, BWD_THREADS, patch_shared_bytes<PATCHES, ZG, SPLITS>(g.patch_columns), s>>>(g, y, xx, epi, a0, a1, \
+                                                                                             acc_in, acc_out)
+        switch (g.bwd_config) {     // patches x stacks of 64 voxels x angle ranges
+        case 1:
+        case 3:
+            if (g.patch_single)
+                CBCT_PATCH(1, false, 1, 8);
+            else if (g.bwd_config == 1)
+                CBCT_PATCH(2, true, 1, 4);
+            else
+                CBCT_PATCH(2, false, 1, 4);
+            break;
+        case 4: CBCT_PATCH(2, true, 2, 2); break;
+        case 5: CBCT_PATCH(2, false, 2, 2); break;
+        case 6: CBCT_PATCH(2, true, 4, 1); break;
+        default: CBCT_PATCH(2, false, 4, 1); break;
         }
 #undef CBCT_PATCH
         return;
