@@ -649,7 +649,7 @@ def run_profile_solve(args):
     (by default 4 rays per lane, 2 x 4 columns x 64 transpose tile; the
     autotuner's choice at this size) and one LSQR solve
     of 2 iterations on a random b, plain launches.  Its first forward_kernel
-    and backward_kernel launches are the instantiations the benchmark's
+    and patch_kernel (transpose) launches are the instantiations the benchmark's
     solvers run (v-fastest projections with the weighted copy, z-fastest
     volume)."""
     import numpy as np

@@ -31,8 +31,9 @@ namespace cbct {
 //
 // Forward and transposed kernels derive every x/y crossing from these tables
 // with the same two rounded operations (plane_alpha); the transpose takes its
-// z crossings from plane_alpha too (zbox), the forward projector from an
-// equivalent one-FMA form measured from the same plane pq.  A^T is the
+// z crossings from plane_alpha too (zbox) or from the row index
+// (patch_crossing), the forward projector from an equivalent one-FMA form
+// measured from the same plane pq.  A^T is the
 // transpose of A; in FP32 the two kernels' segment lengths agree to rounding
 // (not bit for bit), which the dot-product tests bound.
 struct DevGeom {

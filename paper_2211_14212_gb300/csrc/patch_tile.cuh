@@ -17,11 +17,19 @@
 // - Crossings.  Rays only move away from the mid-plane, so a row that enters
 //   its slab k inside the patch does so through the plane nearer to the
 //   mid-plane, and spends the part of [ain, aout] before that crossing in the
-//   neighbouring slab.  That part is summed apart (D, only the first row of a
-//   voxel can have one: the rows that a plane passes between the patch's near
-//   and far depth are at most one, PT_MARGIN included, or two in the general
-//   walk) and moved from voxel to voxel once, after the last angle.  D is a
-//   small part of the sum, so nothing cancels.
+//   neighbouring slab.  That part is summed apart (D) and moved from voxel to
+//   voxel once, after the last angle.  Only a voxel's first row can have one,
+//   as long as a plane passes at most one row between the patch's near and far
+//   depth (PT_MARGIN included); the general walk takes up to PT_CROSSING.  D
+//   is a small part of the sum, so nothing cancels.
+//
+// A^T y at 256^3 / 512^2 / 360 angles: 37.3 ms with backward_tile, 12.6 here;
+// 56 warp instructions per 32 voxels and angle, 63 in the first version
+// (169 in backward_tile), issue slots 76 % busy, 70 % of the sectors from L1.
+// Relative error against FP64 6.8e-7 -> 5.3e-7: fewer and shorter sums.
+// Measured and not kept: prefetching the next column's rows (2.87 against 2.80
+// ms per 90 angles) or the next angle's lines (3.48), four voxels per lane
+// (3.13), four patches per CTA (2.86).
 //
 // Geometries outside patch_columns()'s bounds (steep cones, voxels that cover
 // very many detector columns) take backward_tile.

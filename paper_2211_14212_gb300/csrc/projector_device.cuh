@@ -14,9 +14,9 @@
 // x[j][i][k] so that the lanes of one row group, which sit at ~17 consecutive
 // k of one voxel column, gather one contiguous run.
 //
-// Both projectors take every plane crossing from the per-ray tables of
-// DevGeom (the x/y crossings through plane_alpha in both), so the
-// backprojector is the transpose of the forward projector, not an
+// Both projectors take every x/y plane crossing from the per-ray tables of
+// DevGeom through plane_alpha, and their z crossings from equivalent forms, so
+// the backprojector is the transpose of the forward projector, not an
 // approximation of it (the paper traces Krylov instabilities to unmatched
 // backprojectors, Sec. 2.1.4 and Sec. 4); in FP32 their segment lengths agree
 // to rounding.
@@ -628,7 +628,8 @@ __device__ __forceinline__ void forward_tile(const DevGeom &g, const T *__restri
 
 // ---------------------------------------------------------- transpose A^T y
 //
-// Gather form: each lane owns voxels (i, j, k) of one voxel column and sums
+// The tile for geometries that patch_tile.cuh does not take (steep cones, very
+// coarse voxels) and for the shapes that have no patch form.  Gather form: each lane owns voxels (i, j, k) of one voxel column and sums
 // len * w over every ray that meets them, in registers, angle by angle;
 // the volume is written once (fused epilogue), so there are no atomics and the
 // result does not depend on scheduling.  A warp owns one column (i, j) and
