@@ -102,6 +102,35 @@ k_scale_inplace(float *v, int64_t n, const double *coef, const int *stop) {
         v[i] *= c;
 }
 
+// Step lengths of the conjugate-gradient recursions (CGLS, CGLS-TV).  The
+// vectors are FP32, but alpha and beta act in full.  A step length rounded to
+// FP32 leaves a residual that is not orthogonal to the step: an error along p
+// itself, and p is made mostly of directions the recursion has already solved
+// for, so later steps multiply it.  The roundings of the elements point in no
+// direction and do not grow that way.  CGLS at 32^3, 64^2 pixels, 60 views, 20
+// iterations on noisy data, 32 noise seeds, error of x against FP64: 3.2e-7 to
+// 4.6e-7; with FP32 step lengths 3.3e-7 to 6.2e-6 by the seed.
+//
+// y + c v, c an FP64 scalar as an FP32 pair, rounded once to within the last
+// terms: the product's and the sum's roundings are recovered and added back
+// (two-product and two-sum).  FP32 throughout, since FP64 arithmetic would
+// bound these kernels instead of memory.
+struct ScalarPair {
+    float hi, lo;
+    __host__ __device__ ScalarPair operator-() const { return ScalarPair{-hi, -lo}; }
+};
+// Made by the scalar steps, once: splitting it in every thread of the vector
+// kernels cost 20 iterations of CGLS at 32^3 4 %.
+__host__ __device__ __forceinline__ ScalarPair scalar_pair(double c) {
+    return ScalarPair{(float)c, (float)(c - (double)(float)c)};
+}
+__device__ __forceinline__ float add_scaled(const ScalarPair &c, float v, float y) {
+    const float p = __fmul_rn(c.hi, v), pe = __fmaf_rn(c.hi, v, -p);
+    const float s = __fadd_rn(y, p), b = __fsub_rn(s, y);
+    const float se = __fadd_rn(__fsub_rn(y, __fsub_rn(s, b)), __fsub_rn(p, b));
+    return __fadd_rn(s, __fadd_rn(se, __fmaf_rn(c.lo, v, pe)));
+}
+
 // Combine a basis: x[m] = sum_j coef[j] * basis_j[m], basis_j = basis + j * n.
 // When `stop` is given the launch does nothing once *stop is set (the
 // coefficients of an unfinished step are not valid then).

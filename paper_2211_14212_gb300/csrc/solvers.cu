@@ -240,8 +240,11 @@ struct Reorth {
 //   x += a p;  r -= a q;  s = A^T r - lam^2 x;  gamma' = ||s||^2;
 //   p = s + (gamma'/gamma) p.
 
+// alpha, beta and lam^2 act in full on the FP32 vectors (add_scaled).
+
 struct CgState {
-    double gamma, alpha, beta, lam2;
+    double gamma, lam2;
+    ScalarPair alpha, beta, lam2_pair;
     int iter, stop, status, pad;
 };
 
@@ -272,7 +275,7 @@ cg_after_forward(CgState *st, const double *part_q, int nq, const double *part_p
         st->status = CBCT_EBREAKDOWN;
         return;
     }
-    st->alpha = st->gamma / delta;
+    st->alpha = scalar_pair(st->gamma / delta);
 }
 
 __global__ void __launch_bounds__(RED_THREADS)
@@ -294,7 +297,7 @@ cg_after_backward(CgState *st, const double *part_s, int ns, const double *part_
         st->status = ss == 0.0 ? CBCT_OK : CBCT_EBREAKDOWN;
         return;
     }
-    st->beta = ss / st->gamma;
+    st->beta = scalar_pair(ss / st->gamma);
     st->gamma = ss;
 }
 
@@ -319,10 +322,10 @@ __global__ void __launch_bounds__(VEC_THREADS)
 k_cg_r(float *__restrict__ r, const float *__restrict__ q, int64_t n, double *partial, const CgState *st) {
     __shared__ double red[VEC_THREADS / 32];
     if (st->stop) return;
-    const float a = (float)st->alpha;
+    const ScalarPair a = -st->alpha;
     double s = 0.0;
     for (int64_t i = (int64_t)blockIdx.x * VEC_THREADS + threadIdx.x; i < n; i += (int64_t)VEC_BLOCKS * VEC_THREADS) {
-        const float v = fmaf(-a, q[i], r[i]);
+        const float v = add_scaled(a, q[i], r[i]);
         r[i] = v;
         s += (double)v * v;
     }
@@ -336,12 +339,12 @@ k_cg_xs(float *__restrict__ x, float *__restrict__ s, const float *__restrict__ 
         const CgState *st) {
     __shared__ double red[VEC_THREADS / 32];
     if (st->stop) return;
-    const float a = (float)st->alpha, l2 = (float)st->lam2;
+    const ScalarPair a = st->alpha, l2 = -st->lam2_pair;
     double acc = 0.0;
     for (int64_t i = (int64_t)blockIdx.x * VEC_THREADS + threadIdx.x; i < n; i += (int64_t)VEC_BLOCKS * VEC_THREADS) {
-        const float xi = fmaf(a, p[i], x[i]);
+        const float xi = add_scaled(a, p[i], x[i]);
         x[i] = xi;
-        const float si = fmaf(-l2, xi, s[i]);
+        const float si = add_scaled(l2, xi, s[i]);
         s[i] = si;
         acc += (double)si * si;
     }
@@ -354,10 +357,10 @@ __global__ void __launch_bounds__(VEC_THREADS)
 k_cg_p(float *__restrict__ p, const float *__restrict__ s, int64_t n, double *partial, const CgState *st) {
     __shared__ double red[VEC_THREADS / 32];
     if (st->stop) return;
-    const float b = (float)st->beta;
+    const ScalarPair b = st->beta;
     double acc = 0.0;
     for (int64_t i = (int64_t)blockIdx.x * VEC_THREADS + threadIdx.x; i < n; i += (int64_t)VEC_BLOCKS * VEC_THREADS) {
-        const float v = fmaf(b, p[i], s[i]);
+        const float v = add_scaled(b, p[i], s[i]);
         p[i] = v;
         acc += (double)v * v;
     }
@@ -673,6 +676,7 @@ static cbct_status cgls_solve(const cbct_geometry *geom, const float *b, float *
     };
     CgState init{};
     init.lam2 = o->lambda * o->lambda;
+    init.lam2_pair = scalar_pair(init.lam2);
     CBCT_CUDA_TRY(cudaMemcpyAsync(dst, &init, sizeof init, cudaMemcpyHostToDevice, s));
     const int *stop = &dst->stop;
     int *stopw = &dst->stop;

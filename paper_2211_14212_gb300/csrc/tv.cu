@@ -16,7 +16,8 @@
 namespace cbct {
 
 struct TvState {
-    double gamma, gamma0, alpha, beta, lam;
+    double gamma, gamma0, lam;
+    ScalarPair alpha, beta;
     int iter, stop, pad0, pad1;
 };
 
@@ -135,7 +136,7 @@ k_tv_alpha(TvState *st, const double *part_a, int na, const double *part_d) {
         st->stop = 1;
         return;
     }
-    st->alpha = st->gamma / delta;
+    st->alpha = scalar_pair(st->gamma / delta);
 }
 
 // gamma' = ||s||^2, beta, the history; stop once converged
@@ -152,7 +153,7 @@ k_tv_beta(TvState *st, const double *part_s, const double *part_r, double *hist_
         hist_n[it] = sqrt(g);
     }
     st->iter = it + 1;
-    st->beta = g / st->gamma;
+    st->beta = scalar_pair(g / st->gamma);
     st->gamma = g;
     if (!isfinite(g) || g <= TV_CONVERGED * TV_CONVERGED * st->gamma0) st->stop = 1;
 }
@@ -163,10 +164,10 @@ k_tv_axpy(float *__restrict__ y, const float *__restrict__ x, int64_t n, const T
           double *partial) {
     __shared__ double red[VEC_THREADS / 32];
     if (st->stop) return;
-    const float a = (float)(sign * st->alpha);
+    const ScalarPair a = sign < 0.0 ? -st->alpha : st->alpha;
     double ss = 0.0;
     for (int64_t e = (int64_t)blockIdx.x * VEC_THREADS + threadIdx.x; e < n; e += (int64_t)VEC_BLOCKS * VEC_THREADS) {
-        const float v = fmaf(a, x[e], y[e]);
+        const float v = add_scaled(a, x[e], y[e]);
         y[e] = v;
         ss += (double)v * v;
     }
@@ -180,9 +181,9 @@ k_tv_axpy(float *__restrict__ y, const float *__restrict__ x, int64_t n, const T
 __global__ void __launch_bounds__(VEC_THREADS)
 k_tv_p(float *__restrict__ p, const float *__restrict__ s, int64_t n, const TvState *st, int first) {
     if (!first && st->stop) return;
-    const float b = first ? 0.0f : (float)st->beta;
+    const ScalarPair b = st->beta;
     for (int64_t e = (int64_t)blockIdx.x * VEC_THREADS + threadIdx.x; e < n; e += (int64_t)VEC_BLOCKS * VEC_THREADS)
-        p[e] = first ? s[e] : fmaf(b, p[e], s[e]);
+        p[e] = first ? s[e] : add_scaled(b, p[e], s[e]);
 }
 
 __global__ void k_tv_reset(TvState *st) {
