@@ -124,6 +124,16 @@ static void set_patch_bounds(DevGeom &g, const cbct_geometry_desc &d) {
     g.rho_lo = (float)(rho - g.rho_hi);
     g.m_hi = leading(m);
     g.m_lo = (float)(m - g.m_hi);
+    // A detector with an odd number of rows has one in the mid-plane.  With an
+    // even number of slabs that is the plane between two, and the tables
+    // (axis_map, which A follows) give the row to one of them, by the rounding
+    // of nz / 2 * dz: this transpose has to give it to the same one.
+    g.mid_row = 0.5f * (d.nv - 1);
+    if (d.nv % 2 == 1 && d.nz % 2 == 0) {
+        float f, i, slab;
+        axis_map(0.0, 0.0, -0.5 * d.nz * d.dz, d.dz, d.nz, &f, &i, &slab);
+        if (slab < 0.5f * d.nz) g.mid_row += 0.5f;
+    }
     g.patch_columns = 0;
     // fewer tiles of two patches than two for every SM: halve the tiles and
     // the angles each warp walks (a single A^T y with 23 angles of 40 x 36 x 28
