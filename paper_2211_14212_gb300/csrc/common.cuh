@@ -240,6 +240,9 @@ dim3 backward_grid(const DevGeom &g);
 BrickShape backward_shape(const DevGeom &g);
 // Whether the geometry's configuration runs as patch tiles (patch_tile.cuh).
 bool backward_patches(const DevGeom &g);
+// The default launch shapes of a scan, and the constants of its patch tiles (host only).
+void set_default_shapes(DevGeom &g, const cbct_geometry_desc &d);
 constexpr int NUM_FWD_ROWS = 3, NUM_BWD_CONFIGS = 10;
+constexpr int PT_BOUND_COLUMNS = 22;     // patch tile: most DevGeom::patch_columns
 
 }  // namespace cbct

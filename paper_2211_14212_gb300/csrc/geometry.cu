@@ -151,10 +151,19 @@ static void set_patch_bounds(DevGeom &g, const cbct_geometry_desc &d) {
     // half integers of 12 bits times 11 bits are exact (patch_crossing); a
     // slab covers more than the margins of its planes; 32-bit offsets within
     // a projection; the lists fit 48 KB of shared memory
-    if (columns > 22.0 || passed + 2.0 * 0.05 > 2.95 || rho * far < 0.25 || d.nz > 4096 || d.nv > 4096 || d.nv < 3 ||
+    if (columns > PT_BOUND_COLUMNS || passed + 2.0 * 0.05 > 2.95 || rho * far < 0.25 || d.nz > 4096 || d.nv > 4096 || d.nv < 3 ||
         (int64_t)d.nu * d.nv >= (int64_t)1 << 30)
         return;
     g.patch_columns = std::max(4, (int)columns);
+}
+
+void set_default_shapes(DevGeom &g, const cbct_geometry_desc &d) {
+    g.fwd_rows = d.nv >= 128 ? 4 : d.nv >= 64 ? 2 : 1;   // forward tile: rows per lane by detector height
+    set_patch_bounds(g, d);
+    if (g.patch_columns > 0)
+        g.bwd_config = d.nz > 128 ? 7 : d.nz > 64 ? 5 : 3;   // patch tiles of 256 / 128 / 64 voxels along z
+    else
+        g.bwd_config = d.nz >= 64 ? 3 : 0;   // 2 / 1 voxels per lane by column depth
 }
 }  // namespace cbct
 
@@ -244,7 +253,6 @@ extern "C" cbct_status cbct_geometry_create(const cbct_geometry_desc *d, cbct_ge
         delete g;
         return cuda_fail(err, "cbct_geometry_create");
     }
-    dg.fwd_rows = nv >= 128 ? 4 : nv >= 64 ? 2 : 1;   // forward tile: rows per lane by detector height
     // At most one z-plane crossing per x/y voxel column along every ray: a
     // ray's x/y path inside one column is at most the column's diagonal, and
     // its z slope is at most max|v| / DSD (the pixel farthest from the
@@ -255,11 +263,7 @@ extern "C" cbct_status cbct_geometry_create(const cbct_geometry_desc *d, cbct_ge
         const double zrise = std::sqrt(d->dx * d->dx + d->dy * d->dy) * vmax / d->dsd;
         dg.zsingle = zrise < 0.98 * d->dz ? 1 : 0;
     }
-    set_patch_bounds(dg, *d);
-    if (dg.patch_columns > 0)
-        dg.bwd_config = nz > 128 ? 7 : nz > 64 ? 5 : 3;   // patch tiles of 256 / 128 / 64 voxels along z
-    else
-        dg.bwd_config = nz >= 64 ? 3 : 0;   // 2 / 1 voxels per lane by column depth
+    set_default_shapes(dg, *d);
     dg.angle_block = default_angle_block(dg);
     *out = g;
     return CBCT_OK;

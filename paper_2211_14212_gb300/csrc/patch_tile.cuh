@@ -42,7 +42,7 @@ namespace cbct {
 
 constexpr int PT_ANGLES = 8;             // angles listed at a time, by all splits of a patch together
 constexpr int PT_STEP = 8;               // detector columns listed in one step of a warp (x 4 cells)
-constexpr int PT_MAX_COLUMNS = 24;       // most detector columns across a patch
+constexpr int PT_MAX_COLUMNS = 24;       // PT_BOUND_COLUMNS in steps of PT_STEP
 constexpr float PT_MARGIN = 0.05f;       // pixels; covers the windows' rounding (about 1e-4)
 constexpr int PT_CROSSING = 3;           // most rows that a plane passes between a patch's near and far depth
 constexpr float PT_NEVER = -FLT_MAX;     // crossing alpha of a row that enters its slab before the patch

@@ -41,14 +41,25 @@ constexpr int SRV_MAX_SLOTS = 64;
 constexpr int SRV_FWD_ROWS = 4;                       // forward tile: 4 rays per lane
 constexpr int64_t SRV_SAT_TILES = 2048;                // forward tiles (8 columns x 128 rows) that fill a step
 constexpr int SRV_SRPT_AGE_CAP = 64;                   // SRPT: steps a slot may be passed over before it goes first
-// Transpose tiles: 2 x 4 columns x 64 (configuration 3), or patch tiles of 128
-// voxels along z (configuration 5) for volumes deeper than 64.  A scan whose
-// patches reach more than SRV_COLUMNS detector columns takes the tile that
-// needs no lists: the lists of all CTAs have the size of the largest.
+// Transpose tiles: the patch tiles that set_default_shapes takes for the scan,
+// so that a served iterate is summed like the solver's, and the column tile of
+// configuration 3 where no patch tile applies (column tiles of every shape sum
+// in one order).
 constexpr int SRV_CX = 2, SRV_BK = 2;
-constexpr int SRV_BWD_CONFIG = 3, SRV_BWD_DEEP = 5;
+constexpr int SRV_BWD_CONFIG = 3;
+// The lists of all CTAs of a launch have one size.  A step whose scans have
+// patches of at most SRV_COLUMNS detector columns, the usual case, takes lists
+// of that many (25 KB a CTA); others take the largest (46 KB), which leaves
+// the projections a third of the L1.
 constexpr int SRV_COLUMNS = 12;
-const int SRV_LISTS = std::max(patch_shared_bytes<2, 1, 4>(SRV_COLUMNS), patch_shared_bytes<2, 2, 2>(SRV_COLUMNS));
+static int srv_lists(int columns) {
+    return std::max(std::max(patch_shared_bytes<2, 1, 4>(columns), patch_shared_bytes<2, 2, 2>(columns)),
+                    std::max(patch_shared_bytes<2, 4, 1>(columns), patch_shared_bytes<1, 1, 8>(columns)));
+}
+static void srv_shapes(DevGeom &g) {
+    g.fwd_rows = SRV_FWD_ROWS;
+    if (!backward_patches(g)) g.bwd_config = SRV_BWD_CONFIG;
+}
 
 struct SlotDev {
     DevGeom g;
@@ -143,8 +154,14 @@ __global__ void __launch_bounds__(BWD_THREADS, 4) srv_backward(const SlotTable *
         if (g_sh.patch_columns == 0)
             backward_tile<float, true, SRV_CX, SRV_BK, 2>(g_sh, sd.Uw, sd.V, epi, tbx, tby, tbz, 0, g_sh.nangles,
                                                           nullptr, nullptr, partial_at);
-        else if (g_sh.bwd_config == SRV_BWD_DEEP)
+        else if (g_sh.bwd_config == 7)
+            patch_tile<float, true, 2, false, 4, 1>(g_sh, sd.Uw, sd.V, epi, tbx, tby, tbz, 0, g_sh.nangles, nullptr,
+                                                 nullptr, partial_at, (char *)patch_lists);
+        else if (g_sh.bwd_config == 5)
             patch_tile<float, true, 2, false, 2, 2>(g_sh, sd.Uw, sd.V, epi, tbx, tby, tbz, 0, g_sh.nangles, nullptr,
+                                                 nullptr, partial_at, (char *)patch_lists);
+        else if (g_sh.patch_single)
+            patch_tile<float, true, 1, false, 1, 8>(g_sh, sd.Uw, sd.V, epi, tbx, tby, tbz, 0, g_sh.nangles, nullptr,
                                                  nullptr, partial_at, (char *)patch_lists);
         else
             patch_tile<float, true, 2, false, 1, 4>(g_sh, sd.Uw, sd.V, epi, tbx, tby, tbz, 0, g_sh.nangles, nullptr,
@@ -240,25 +257,18 @@ struct Slot {
     cudaGraphExec_t solo_graph = nullptr;   // captured step of this slot alone (enqueue_step)
 };
 
-// Forward tiles and bricks of a scan under the server's launch shapes (the
-// deep transpose tiles are fewer).
-void grids(const cbct_geometry_desc &d, int &fgx, int &fgy, int &bgx, int &bgy, int &bgz) {
-    fgx = (d.nu + FWD_COLS - 1) / FWD_COLS;
-    fgy = (d.nv + 32 * SRV_FWD_ROWS - 1) / (32 * SRV_FWD_ROWS);
-    bgx = (d.nx + SRV_CX - 1) / SRV_CX;
-    bgy = (d.ny + (8 / SRV_CX) - 1) / (8 / SRV_CX);
-    bgz = (d.nz + 32 * SRV_BK - 1) / (32 * SRV_BK);
-}
-
 // Device memory a request holds at its peak (ray tables, Krylov vectors,
 // staging of b, partial sums, state and histories), rounded up per buffer.
 size_t request_bytes(const cbct_geometry_desc &d, int method, int iters) {
     auto al = [](size_t b) { return (b + 1023) & ~(size_t)1023; };
     // m: a volume-side vector in the padded z-fastest layout
     const size_t n = (size_t)d.nangles * d.nv * d.nu, m = (size_t)d.nx * d.ny * (d.nz + 2) + 2 * ZF_GUARD;
-    int fgx, fgy, bgx, bgy, bgz;
-    grids(d, fgx, fgy, bgx, bgy, bgz);
-    const size_t nf = (size_t)fgx * fgy * d.nangles, nb = (size_t)bgx * bgy * bgz;
+    DevGeom g{};                                            // what the tile grids depend on
+    g.nx = d.nx; g.ny = d.ny; g.nz = d.nz; g.nu = d.nu; g.nv = d.nv; g.nangles = d.nangles;
+    set_default_shapes(g, d);
+    srv_shapes(g);
+    const dim3 fg = forward_grid(g), bg = backward_grid(g);
+    const size_t nf = (size_t)fg.x * fg.y * fg.z, nb = (size_t)bg.x * bg.y * bg.z;
     size_t t = al((size_t)d.nangles * d.nu * 24) + al((size_t)d.nv * 16) + al(n / d.nangles * 4) + al(d.nangles * 8);
     t += al((size_t)d.nz * d.nv * 8);                       // z slab table
     t += 3 * al(n * 4);                                     // U, |d'| U and the staged b
@@ -312,8 +322,10 @@ struct ServerImpl {
     std::vector<Slot> slots;
     std::vector<int> step_slots;      // slots advanced by the current step, in slot-table order
     bool table_dirty = true;
-    cudaGraphExec_t step_graph = nullptr;
-    int fwd_grid = 0, bwd_grid = 0, vec_grid = 0;
+    // [1]: steps with a scan of more than SRV_COLUMNS columns across a patch
+    cudaGraphExec_t step_graph[2] = {nullptr, nullptr};
+    int bwd_grid[2] = {0, 0}, lists[2] = {0, 0};
+    int fwd_grid = 0, vec_grid = 0;
     int64_t steps_run = 0, graph_replays = 0;
 
     void run_admission();
@@ -339,10 +351,7 @@ cbct_status ServerImpl::setup_slot(Slot &sl) {
     r.desc.angles_rad = r.angles.data();
     cbct_status st = cbct_geometry_create(&r.desc, &sl.geom);
     if (st != CBCT_OK) return st;
-    sl.geom->dev.fwd_rows = SRV_FWD_ROWS;
-    sl.geom->dev.patch_single = 0;          // one tile shape per depth, as srv_backward has them
-    if (sl.geom->dev.patch_columns > SRV_COLUMNS) sl.geom->dev.patch_columns = 0;
-    sl.geom->dev.bwd_config = sl.geom->dev.patch_columns > 0 && sl.geom->dev.nz > 64 ? SRV_BWD_DEEP : SRV_BWD_CONFIG;
+    srv_shapes(sl.geom->dev);
     const DevGeom &g = sl.geom->dev;
     // m: a volume-side vector in the padded z-fastest layout (pads zeroed below)
     const int64_t n = cbct_geometry_num_rays(sl.geom), m = zf_len(g);
@@ -494,6 +503,8 @@ void ServerImpl::return_budget(const std::shared_ptr<Request> &r) {
 // bit for bit.  That step is captured once per slot.
 cbct_status ServerImpl::enqueue_step() {
     Slot *solo = solo_step() ? &slots[step_slots[0]] : nullptr;
+    int wide = 0;
+    for (int i : step_slots) wide |= slots[i].geom->dev.patch_columns > SRV_COLUMNS;
     auto launch_all = [&]() -> cudaError_t {
         if (solo) {
             const DevGeom &g = solo->geom->dev;
@@ -515,7 +526,7 @@ cbct_status ServerImpl::enqueue_step() {
             if (e0 != cudaSuccess) return e0;
             srv_forward<<<fwd_grid, FWD_THREADS, 0, s>>>(tab_dev, counters);
             srv_after_forward<<<SRV_MAX_SLOTS, RED_THREADS, 0, s>>>(tab_dev);
-            srv_backward<<<bwd_grid, BWD_THREADS, SRV_LISTS, s>>>(tab_dev, counters + 1);
+            srv_backward<<<bwd_grid[wide], BWD_THREADS, lists[wide], s>>>(tab_dev, counters + 1);
             srv_after_backward<<<SRV_MAX_SLOTS, RED_THREADS, 0, s>>>(tab_dev);
         }
         srv_update<<<vec_grid, VEC_THREADS, 0, s>>>(tab_dev);
@@ -525,7 +536,7 @@ cbct_status ServerImpl::enqueue_step() {
             e = cudaMemcpyAsync(stat_host, stat_dev, sizeof(SlotStatus) * SRV_MAX_SLOTS, cudaMemcpyDeviceToHost, s);
         return e;
     };
-    cudaGraphExec_t &exec = solo ? solo->solo_graph : step_graph;
+    cudaGraphExec_t &exec = solo ? solo->solo_graph : step_graph[wide];
     if (use_graph && !exec) {
         cudaGraph_t graph = nullptr;
         cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
@@ -832,10 +843,14 @@ extern "C" cbct_status cbct_server_create(const cbct_server_opts *o, cbct_server
     S.schedule = o->schedule;
     S.t0 = std::chrono::steady_clock::now();
     cudaError_t e = cudaGetDevice(&S.device);
-    int sms = 0, occ_f = 0, occ_b = 0;
+    int sms = 0, occ_f = 0, occ_b[2] = {0, 0};
+    S.lists[0] = srv_lists(SRV_COLUMNS);
+    S.lists[1] = srv_lists(PT_BOUND_COLUMNS);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, S.device);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_f, srv_forward, FWD_THREADS, 0);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_b, srv_backward, BWD_THREADS, SRV_LISTS);
+    for (int w = 0; w < 2; ++w)
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_b[w], srv_backward, BWD_THREADS, S.lists[w]);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&S.s, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&S.s_admit, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&S.s_read, cudaStreamNonBlocking);
@@ -852,7 +867,7 @@ extern "C" cbct_status cbct_server_create(const cbct_server_opts *o, cbct_server
     }
     std::memset(S.tab_host, 0, sizeof(SlotTable));
     S.fwd_grid = sms * std::max(occ_f, 1);
-    S.bwd_grid = sms * std::max(occ_b, 1);
+    for (int w = 0; w < 2; ++w) S.bwd_grid[w] = sms * std::max(occ_b[w], 1);
     S.vec_grid = sms * 4;
     try {
         S.reader = std::thread([&S] { S.run_readout(); });
@@ -1018,7 +1033,8 @@ extern "C" void cbct_server_destroy(cbct_server *srv) {
     S.ready.clear();
     for (cbct_geometry *g : S.graveyard) cbct_geometry_destroy(g);
     S.graveyard.clear();
-    if (S.step_graph) cudaGraphExecDestroy(S.step_graph);
+    for (cudaGraphExec_t exec : S.step_graph)
+        if (exec) cudaGraphExecDestroy(exec);
     for (cudaStream_t st : {S.s, S.s_admit, S.s_read}) cudaStreamSynchronize(st);
     free_server_resources(S);
     delete srv;
