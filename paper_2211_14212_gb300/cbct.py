@@ -325,7 +325,9 @@ def get_angle_block(geom: Geometry) -> int:
     return int(a.value)
 
 
-TUNE_CACHE_VERSION = 1
+# Raised whenever other kernels run behind the same shapes: a choice timed with
+# the old ones says nothing about the new ones (2: the patch tiles).
+TUNE_CACHE_VERSION = 2
 
 
 def tune_key(params: dict, nangles: int, device: str) -> str:
@@ -347,7 +349,7 @@ def tune_key(params: dict, nangles: int, device: str) -> str:
 
 class TuneCache:
     """Launch shapes chosen by `autotune`, per geometry class, in a JSON file
-    {"version": 1, "entries": {key: {"fwd_rows", "bwd_config", ...}}}.  A
+    {"version": 2, "entries": {key: {"fwd_rows", "bwd_config", ...}}}.  A
     missing, unreadable or other-version file reads as empty; `put` merges
     with what is on disk and replaces the file atomically."""
 
