@@ -115,6 +115,11 @@ static float leading(double v) {
     return (float)std::ldexp(std::nearbyint(f * 2048.0), e - 11);
 }
 
+// Tiles of two patches and `depth` voxels along z.
+static int64_t patch_tiles(const cbct_geometry_desc &d, int depth) {
+    return (int64_t)((d.nx + 1) / 2) * ((d.ny + 3) / 4) * ((d.nz + depth - 1) / depth);
+}
+
 // Where the patch tile applies (patch_tile.cuh), and its constants: bounds of
 // a patch's footprint over every position and angle.
 static void set_patch_bounds(DevGeom &g, const cbct_geometry_desc &d) {
@@ -138,7 +143,7 @@ static void set_patch_bounds(DevGeom &g, const cbct_geometry_desc &d) {
     // fewer tiles of two patches than two for every SM: halve the tiles and
     // the angles each warp walks (a single A^T y with 23 angles of 40 x 36 x 28
     // voxels: 26.7 -> 21.4 us)
-    g.patch_single = d.nz <= 64 && (int64_t)((d.nx + 1) / 2) * ((d.ny + 3) / 4) < 304;
+    g.patch_single = patch_tiles(d, 64) < 304;
     // a patch may reach one voxel out of the volume
     const double r = std::hypot((0.5 * d.nx + 1.0) * d.dx, (0.5 * d.ny + 1.0) * d.dy);
     if (r >= 0.95 * d.dso) return;
@@ -160,8 +165,15 @@ static void set_patch_bounds(DevGeom &g, const cbct_geometry_desc &d) {
 void set_default_shapes(DevGeom &g, const cbct_geometry_desc &d) {
     g.fwd_rows = d.nv >= 128 ? 4 : d.nv >= 64 ? 2 : 1;   // forward tile: rows per lane by detector height
     set_patch_bounds(g, d);
+    // Patch tiles of 256 / 128 / 64 voxels along z: the deeper ones list the
+    // columns for more voxels but split the angles over fewer warps, and pay
+    // from 512 tiles on (A^T y of 180 angles, 256 / 128 / 64 deep: 64 x 64 x 200
+    // voxels 528 / 562 / 617 us, 40 x 40 x 200 365 / 254 / 288, 8 x 8 x 200 332 /
+    // 210 / 88; with the column tiles 1250, 558 and 217).
     if (g.patch_columns > 0)
-        g.bwd_config = d.nz > 128 ? 7 : d.nz > 64 ? 5 : 3;   // patch tiles of 256 / 128 / 64 voxels along z
+        g.bwd_config = d.nz > 128 && patch_tiles(d, 256) >= 512  ? 7
+                       : d.nz > 64 && patch_tiles(d, 128) >= 512 ? 5
+                                                                 : 3;
     else
         g.bwd_config = d.nz >= 64 ? 3 : 0;   // 2 / 1 voxels per lane by column depth
 }

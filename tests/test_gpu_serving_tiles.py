@@ -40,13 +40,15 @@ def geom(nx, ny, nz, vox, nu, nv, pix, dso=1000.0, dsd=1536.0, angles=40):
     return synth.Geometry(nx, ny, nz, vox, vox, vox, nu, nv, pix, pix, dso, dsd, synth.circular_angles(angles) + 0.003)
 
 
-# one patch a tile; two; two stacks; four stacks; more than 12 columns across a
-# patch; a steep cone, which no patch tile takes
+# one patch a tile; two; two stacks; four stacks; one patch and several tiles
+# along z; more than 12 columns across a patch; a steep cone, which no patch
+# tile takes
 SCANS = {
     "small": geom(20, 18, 24, 8.0, 40, 48, 8.0),
     "stack_64": geom(52, 50, 40, 5.0, 80, 70, 5.0),
-    "stacks_70": geom(24, 22, 70, 3.0, 50, 160, 2.5),
-    "stacks_130": geom(14, 12, 130, 2.0, 40, 290, 1.5),
+    "stacks_70": geom(64, 64, 70, 3.0, 110, 150, 3.0),
+    "stacks_130": geom(64, 64, 130, 2.0, 110, 230, 2.0),
+    "deep_small": geom(14, 12, 130, 2.0, 40, 290, 1.5),
     "columns_17": geom(24, 20, 30, 8.0, 300, 70, 1.5 * 8.0 * 1.536 / 8.2),
     "steep": geom(20, 20, 30, 2.0, 40, 60, 6.0, dso=45.0, dsd=120.0),
 }
