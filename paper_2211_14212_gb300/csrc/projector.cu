@@ -22,8 +22,14 @@ namespace cbct {
 // A x at 512^3 / 768 x 512 / 180 angles: 4 rays 23.5 ms with 4 cells and 2
 // CTAs, 31.6 ms with 2 cells and 3; 2 rays 26.3 ms with 8 cells and 3 CTAs,
 // 29.6 ms with 4 cells and 4.
-template <typename T, bool COMP, int R, bool VF, bool OFF32>
-__global__ void __launch_bounds__(FWD_THREADS, R >= 4 ? 2 : R == 2 ? 3 : 4)
+// Steep cones have a kernel without the cell walk (CELLS): the crossing-by-
+// crossing walk keeps few loads in flight and takes the warps instead.  A x at
+// 96^3 / 150 x 300 / 90 angles under a steep cone: 844 us in the kernel of both
+// walks, 640 here.  The other way round it does not pay: without the second
+// walk the cell walk was scheduled worse (FP32 256^3 12.9 -> 13.0 ms, FP16 512^3
+// 20.6 -> 22.6).
+template <typename T, bool COMP, int R, bool VF, bool OFF32, bool CELLS>
+__global__ void __launch_bounds__(FWD_THREADS, CELLS ? (R >= 4 ? 2 : R == 2 ? 3 : 4) : R >= 4 ? 3 : 4)
 forward_kernel(DevGeom g, const T *__restrict__ vol, T *__restrict__ proj, Epilogue epi) {
     __shared__ float4 lists[FWD_COLS * FWD_LIST];
     if (epi.stop && *epi.stop) return;
@@ -31,7 +37,7 @@ forward_kernel(DevGeom g, const T *__restrict__ vol, T *__restrict__ proj, Epilo
         const size_t b = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
         return epi.partial ? epi.partial + b * TILE_PARTIALS : nullptr;
     };
-    forward_tile<T, COMP, R, VF, OFF32>(g, vol, proj, epi, blockIdx.x, blockIdx.z, blockIdx.y, partial_at, lists);
+    forward_tile<T, COMP, R, VF, OFF32, CELLS>(g, vol, proj, epi, blockIdx.x, blockIdx.z, blockIdx.y, partial_at, lists);
 }
 
 template <int R>
@@ -71,24 +77,26 @@ int forward_num_blocks(const DevGeom &g) {
 // about 1023^3 voxels is larger).
 constexpr uint64_t OFF32_BYTES = (uint64_t)1 << 32;
 
+template <typename T, bool COMP, int R, bool VF>
+static void launch_forward_t(const DevGeom &g, const void *x, void *y, const Epilogue &epi, cudaStream_t s) {
+    const dim3 grid = forward_grid(g);
+    const T *xx = (const T *)x;
+    T *yy = (T *)y;
+    if (!g.zsingle)
+        forward_kernel<T, COMP, R, VF, true, false><<<grid, FWD_THREADS, 0, s>>>(g, xx, yy, epi);
+    else if (sizeof(T) == 2 || (uint64_t)zf_len(g) * sizeof(T) <= OFF32_BYTES)   // 16 bits: at most 2^31 elements
+        forward_kernel<T, COMP, R, VF, true, true><<<grid, FWD_THREADS, 0, s>>>(g, xx, yy, epi);
+    else if constexpr (sizeof(T) != 2)
+        forward_kernel<T, COMP, R, VF, false, true><<<grid, FWD_THREADS, 0, s>>>(g, xx, yy, epi);
+}
+
 template <int R, bool VF>
 static void launch_forward_r(const DevGeom &g, const void *x, void *y, cbct_dtype t, const Epilogue &epi,
                              cudaStream_t s) {
-    const dim3 grid = forward_grid(g);
     switch (t) {
-    case CBCT_F32:
-        if ((uint64_t)zf_len(g) * sizeof(float) <= OFF32_BYTES)
-            forward_kernel<float, false, R, VF, true><<<grid, FWD_THREADS, 0, s>>>(g, (const float *)x, (float *)y, epi);
-        else
-            forward_kernel<float, false, R, VF, false><<<grid, FWD_THREADS, 0, s>>>(g, (const float *)x, (float *)y, epi);
-        break;
-    case CBCT_F16:                  // at most 2^31 elements (validate_geometry_desc)
-        forward_kernel<__half, true, R, VF, true><<<grid, FWD_THREADS, 0, s>>>(g, (const __half *)x, (__half *)y, epi);
-        break;
-    case CBCT_BF16:
-        forward_kernel<__nv_bfloat16, true, R, VF, true><<<grid, FWD_THREADS, 0, s>>>(
-            g, (const __nv_bfloat16 *)x, (__nv_bfloat16 *)y, epi);
-        break;
+    case CBCT_F32: launch_forward_t<float, false, R, VF>(g, x, y, epi, s); break;
+    case CBCT_F16: launch_forward_t<__half, true, R, VF>(g, x, y, epi, s); break;
+    case CBCT_BF16: launch_forward_t<__nv_bfloat16, true, R, VF>(g, x, y, epi, s); break;
     }
 }
 

@@ -574,13 +574,14 @@ __device__ __forceinline__ void trace_rays_zsingle(const DevGeom &g, const T *__
 // the epilogue, so that the address it computes is not held in a register
 // through the traversal, and the sums need no block barrier (measured 6 %
 // of the transpose's time with one).
+// CELLS: the cell walk is compiled in (taken where DevGeom::zsingle).
 
 // lists: FWD_COLS * FWD_LIST float4 of shared memory (the warps' cell lists).
 
 constexpr int FWD_COLS = 8, FWD_THREADS = 32 * FWD_COLS;
 constexpr int FWD_LIST = CELL_CHUNK / 2;         // float4 of one warp's cell list
 
-template <typename T, bool COMP, int R, bool VFAST, bool OFF32, typename PartialAt>
+template <typename T, bool COMP, int R, bool VFAST, bool OFF32, bool CELLS, typename PartialAt>
 __device__ __forceinline__ void forward_tile(const DevGeom &g, const T *__restrict__ vol, T *__restrict__ proj,
                                              const Epilogue &epi, int tx, int ty, int a, PartialAt &&partial_at,
                                              float4 *lists) {
@@ -594,7 +595,7 @@ __device__ __forceinline__ void forward_tile(const DevGeom &g, const T *__restri
     if (col_ok) {
         RayAxis rx, ry, rz[R];
         load_rays<R>(g, a, iu, iv0, g.nv, rx, ry, rz);
-        if (g.zsingle) {
+        if (CELLS && g.zsingle) {
             trace_rays_zsingle<T, COMP, R, OFF32>(g, vol, rx, ry, rz, lists + warp * FWD_LIST, acc);
         } else {
             // several z crossings per xy cell are possible: the exact

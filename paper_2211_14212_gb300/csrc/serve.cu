@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) srv_forward(const SlotTable *t
         const int local = item - tab->fwd_start[s];
         const int tx = local % sd.fgx, a = (local / sd.fgx) % g_sh.nangles, ty = local / (sd.fgx * g_sh.nangles);   // as forward_grid
         const Epilogue epi{&sd.st->fa, &sd.st->fb, 0.0, 0.0, nullptr, nullptr, nullptr, sd.Uw};
-        forward_tile<float, false, SRV_FWD_ROWS, true, false>(g_sh, sd.V, sd.U, epi, tx, ty, a,
+        forward_tile<float, false, SRV_FWD_ROWS, true, false, true>(g_sh, sd.V, sd.U, epi, tx, ty, a,
                                                        [&]() { return sd.pf + (size_t)local * TILE_PARTIALS; }, lists);
     }
 }
