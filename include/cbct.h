@@ -101,7 +101,10 @@ cbct_status cbct_project(const cbct_geometry *geom, const void *x, void *y,
  * the same crossing tables, so <A x, y> = <x, A^T y> up to FP32 rounding of
  * the lengths and sums; Sec. 2.1.4 explains why an unmatched backprojector
  * breaks the Krylov methods).  y: N device
- * elements, x: M device elements of `dtype`.  Asynchronous on `stream`. */
+ * elements, x: M device elements of `dtype`.  Asynchronous on `stream`.
+ * Neighbouring rows enter a voxel's sum with weight 0, so a non-finite value
+ * in y makes the voxels along its ray, and up to three slabs beside them, NaN
+ * or infinite. */
 cbct_status cbct_backproject(const cbct_geometry *geom, const void *y, void *x,
                              cbct_dtype dtype, cbct_stream stream);
 
@@ -138,16 +141,24 @@ cbct_status cbct_backproject_voxel_driven(const cbct_geometry *geom, const float
 cbct_status cbct_count_nnz(const cbct_geometry *geom, int64_t *nnz, cbct_stream stream);
 
 /* Launch shapes of the projectors of one geometry (performance only: every
- * shape computes the same A and A^T).  fwd_rows: rays per lane of the forward
- * tile (1, 2 or 4; a warp follows 32 * fwd_rows rows of one detector column).
- * bwd_config: tile of the transpose (one warp per voxel column), 0 = 4 x 2
- * columns x 32 voxels along z (1 per lane), 1 = 4 x 2 x 64 (2 per lane),
- * 2 = 8 x 1 x 32, 3 = 2 x 4 x 64, 4 = 4 x 2 x 128 (4 per lane),
- * 5 = 2 x 4 x 128, 6 = 4 x 2 x 256 (8 per lane), 7 = 2 x 4 x 256,
- * 8 = 2 x 4 x 128 and 9 = 4 x 2 x 128 holding each voxel's candidate rows in
- * registers per angle (configurations 0..3 do too; 4..7 re-read them per
- * detector column).  Changing the shape while another thread uses the
- * geometry is a data race. */
+ * shape computes the same A and A^T, up to the order of the FP32 sums).
+ * fwd_rows: rays per lane of the forward tile (1, 2 or 4; a warp follows
+ * 32 * fwd_rows rows of one detector column); it does not change the sums.
+ * bwd_config: tile of the transpose in voxel columns (x by y) and voxels along
+ * z.  1 = 4 x 2 x 64, 3 = 2 x 4 x 64, 4 = 4 x 2 x 128, 5 = 2 x 4 x 128,
+ * 6 = 4 x 2 x 256 and 7 = 2 x 4 x 256 are patch tiles (a warp sums 2 x 2
+ * columns x 64 voxels, and the shallower tiles split the angles into 2, 4 or,
+ * for volumes of few tiles, 8 ranges); they differ in the last bits.
+ * 0 = 4 x 2 x 32, 2 = 8 x 1 x 32, 8 = 2 x 4 x 128 and 9 = 4 x 2 x 128 are column
+ * tiles (a warp sums one column), which all give the same bits.  Where no
+ * patch tile applies (steep cones, voxels that cover very many pixels, less
+ * than 3 rows) 1 and 3 run as column tiles of their shape, 4, 6 as 9 and 5, 7
+ * as 8.  The default is 3, 5 or 7 by the volume's depth and number of tiles (0
+ * or 3 without patch tiles).  Late iterates of ill-conditioned problems
+ * amplify differences of the last bits (4e-3 relative after 20 to 40
+ * iterations has been seen), so a solve repeats bit for bit only at the same
+ * shape: autotuning picks by time.  Changing the shape while another thread
+ * uses the geometry is a data race. */
 #define CBCT_TUNE_TIMES 13
 cbct_status cbct_geometry_set_launch(cbct_geometry *geom, int fwd_rows, int bwd_config);
 cbct_status cbct_geometry_get_launch(const cbct_geometry *geom, int *fwd_rows, int *bwd_config);
@@ -166,9 +177,10 @@ cbct_status cbct_geometry_autotune(cbct_geometry *geom, int max_angles, double *
  * `angles` consecutive angles, keeping FP32 running sums in M values of
  * scratch, so that each pass gathers from projections that stay in L2.
  * angles >= nangles means one pass; angles == 0 restores the default (one
- * pass); negative values are rejected (CBCT_EINVAL).  Every block size gives
- * bit-identical sums (the running sums are kept in FP32 between passes, in
- * the same order).  Not thread-safe, like set_launch. */
+ * pass); negative values are rejected (CBCT_EINVAL).  The running sums are kept
+ * in FP32 between passes: column tiles (set_launch) give the same bits for
+ * every block size, patch tiles, which split each pass's angles into ranges,
+ * the same sums up to FP32 rounding.  Not thread-safe, like set_launch. */
 cbct_status cbct_geometry_set_angle_block(cbct_geometry *geom, int angles);
 cbct_status cbct_geometry_get_angle_block(const cbct_geometry *geom, int *angles);
 
@@ -321,11 +333,11 @@ cbct_status cbct_hybrid_lsmr_solve(const cbct_geometry *geom, const float *b, fl
  * CBCT_SCHED_RATIO orders them by response ratio (age + remaining time) /
  * remaining time (remaining time from the same cost model and the measured
  * work rate); CBCT_SCHED_SHARE advances every admitted request every step.
- * Each result equals the single-request solver's up to FP32 rounding: the
- * server's tiles sum every ray and voxel in the same order, but a single
- * request tuned to other launch shapes (cbct_geometry_autotune) sums its norm
- * partials in other groups, and late iterates of ill-conditioned problems
- * amplify such differences (about 1e-4 relative after 20-40 iterations).
+ * Each result equals the single-request solver's at the default launch shapes
+ * up to FP32 rounding: the server's tiles sum every ray and voxel in the same
+ * order.  A single request at other shapes (cbct_geometry_autotune) sums in
+ * another one, and late iterates of ill-conditioned problems amplify such
+ * differences (see cbct_geometry_set_launch).
  * Requests use FP32 storage and LSQR or LSMR.  All calls are thread-safe
  * except cbct_server_destroy, which must not overlap any other call on the
  * same server. */

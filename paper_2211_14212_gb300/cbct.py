@@ -297,6 +297,8 @@ def count_nnz(geom: Geometry, stream=None) -> int:
 
 TUNE_TIMES = 13
 FWD_ROWS = (1, 2, 4)
+# Names of the transpose tiles (cbct_geometry_set_launch says which kernel each
+# runs; without patch tiles the 256-deep ones are 128 deep).
 BWD_CONFIGS = ("4x2 columns x 32", "4x2 columns x 64", "8x1 columns x 32", "2x4 columns x 64",
                "4x2 columns x 128", "2x4 columns x 128", "4x2 columns x 256", "2x4 columns x 256",
                "2x4 columns x 128, rows held", "4x2 columns x 128, rows held")

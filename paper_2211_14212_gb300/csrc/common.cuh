@@ -53,7 +53,7 @@ struct DevGeom {
     int fwd_rows;            // forward tile: rays per lane (1, 2 or 4)
     int bwd_config;          // transpose tile (backward_shape)
     int patch_columns;       // patch tile: most detector columns across a patch, 0 when it does not apply
-    int patch_single;        // configurations 1 and 3: tiles of one patch and 8 angle ranges
+    int patch_single;        // configurations 1 and 3 run as tiles of one patch and 8 angle ranges
     float rho, rho_hi, rho_lo;   // dz / dv, and its leading 11 bits and the rest
     float m_hi, m_lo;        // the same for dso / dsd
     float mid_row;           // patch tile: rows from here on lie above the mid-plane (set_patch_bounds)

@@ -31,8 +31,8 @@
 // ms per 90 angles) or the next angle's lines (3.48), four voxels per lane
 // (3.13), four patches per CTA (2.86).
 //
-// Geometries outside patch_columns()'s bounds (steep cones, voxels that cover
-// very many detector columns) take backward_tile.
+// Geometries outside the bounds of set_patch_bounds (steep cones, voxels that
+// cover very many detector columns) take backward_tile.
 #pragma once
 
 #include "projector_device.cuh"

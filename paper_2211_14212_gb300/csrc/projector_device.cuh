@@ -646,11 +646,12 @@ __device__ __forceinline__ void forward_tile(const DevGeom &g, const T *__restri
 // ---------------------------------------------------------- transpose A^T y
 //
 // The tile for geometries that patch_tile.cuh does not take (steep cones, very
-// coarse voxels) and for the shapes that have no patch form.  Gather form: each lane owns voxels (i, j, k) of one voxel column and sums
-// len * w over every ray that meets them, in registers, angle by angle;
-// the volume is written once (fused epilogue), so there are no atomics and the
-// result does not depend on scheduling.  A warp owns one column (i, j) and
-// 32 K consecutive k (k = k0 + kk * 32 + lane); a tile is 8 warps on a
+// coarse voxels) and for the shapes that have no patch form.  Gather form:
+// each lane owns voxels (i, j, k) of one voxel column and sums len * w over
+// every ray that meets them, in registers, angle by angle; the volume is
+// written once (fused epilogue), so there are no atomics and the result does
+// not depend on scheduling.  A warp owns one column (i, j) and 32 K consecutive
+// k (k = k0 + kk * 32 + lane); a tile is 8 warps on a
 // CX x (8 / CX) patch of columns.  For every angle the warp projects the
 // cell's four corners to find the detector columns whose xy projection
 // crosses cell (i, j), and each lane the detector rows that can meet its
