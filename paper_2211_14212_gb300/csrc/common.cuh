@@ -56,7 +56,7 @@ struct DevGeom {
     int patch_single;        // configurations 1 and 3 run as tiles of one patch and 8 angle ranges
     float rho, rho_hi, rho_lo;   // dz / dv, and its leading 11 bits and the rest
     float m_hi, m_lo;        // the same for dso / dsd
-    float mid_row;           // patch tile: rows from here on lie above the mid-plane (set_patch_bounds)
+    float mid_down;          // patch tile: > 0 when the middle row belongs to the slab below the mid-plane (set_patch_bounds)
     int angle_block;         // transpose: angles per pass when summed in passes (launch_backward)
 };
 

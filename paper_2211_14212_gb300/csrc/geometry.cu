@@ -133,11 +133,11 @@ static void set_patch_bounds(DevGeom &g, const cbct_geometry_desc &d) {
     // even number of slabs that is the plane between two, and the tables
     // (axis_map, which A follows) give the row to one of them, by the rounding
     // of nz / 2 * dz: this transpose has to give it to the same one.
-    g.mid_row = 0.5f * (d.nv - 1);
+    g.mid_down = 0.0f;
     if (d.nv % 2 == 1 && d.nz % 2 == 0) {
         float f, i, slab;
         axis_map(0.0, 0.0, -0.5 * d.nz * d.dz, d.dz, d.nz, &f, &i, &slab);
-        if (slab < 0.5f * d.nz) g.mid_row += 0.5f;
+        if (slab < 0.5f * d.nz) g.mid_down = 1e-30f;     // patch_crossing
     }
     g.patch_columns = 0;
     // fewer tiles of two patches than two for every SM: halve the tiles and
