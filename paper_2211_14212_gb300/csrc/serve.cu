@@ -387,12 +387,13 @@ cbct_status ServerImpl::setup_slot(Slot &sl) {
     init.sqrt_m = std::sqrt((double)cbct_geometry_num_voxels(sl.geom));
     if (e == cudaSuccess) e = cudaMemcpyAsync(sl.st, &init, sizeof init, cudaMemcpyHostToDevice, sa);
     if (e != cudaSuccess) return cuda_fail(e, "server: slot allocation");
-    // beta_1 u_1 = b, alpha_1 v_1 = A^T u_1: the same start as the single-request solver
-    k_sumsq<float><<<VEC_BLOCKS, VEC_THREADS, 0, sa>>>(sl.b, n, sl.pf);
-    gk_begin<<<1, RED_THREADS, 0, sa>>>(sl.st, sl.pf, VEC_BLOCKS);
-    // U = su * b, v-fastest
+    // beta_1 u_1 = b, alpha_1 v_1 = A^T u_1: the same start as the single-request solver,
+    // ||b||^2 included, which is summed in the v-fastest layout
     st = launch_proj_relayout(g, sl.b, sl.U, CBCT_F32, true, sa);
     if (st != CBCT_OK) return st;
+    k_sumsq<float><<<VEC_BLOCKS, VEC_THREADS, 0, sa>>>(sl.U, n, sl.pf);
+    gk_begin<<<1, RED_THREADS, 0, sa>>>(sl.st, sl.pf, VEC_BLOCKS);
+    // U = su * b
     k_scale_inplace<<<VEC_BLOCKS, VEC_THREADS, 0, sa>>>(sl.U, n, &sl.st->c0, &sl.st->stop);
     st = launch_weight(g, sl.U, CBCT_F32, sl.Uw, sa);
     if (st != CBCT_OK) return st;

@@ -85,9 +85,11 @@ def test_mixed_step_equals_solver(cbct, problems, iters):
     synth.Geometry(40, 40, 150, 2.0, 2.0, 2.0, 128, 400, 1.2, 1.2, 1000.0, 1536.0, synth.circular_angles(90))],
     ids=["128", "columns_above_12", "stacks_150"])
 def test_step_of_one_scan_equals_solver(cbct, g):
-    """Scans that fill a step alone: the single-request kernels, captured."""
+    """Scans that fill a step alone: the single-request kernels, captured, from
+    the same start, so every bit is the solver's, the FP64 norms included."""
     b = data(g, 90)
     with cbct.Server(16 << 30, max_slots=4) as srv:
-        x = srv.wait(srv.submit(g, b, "lsqr", 30), timeout=300).x
-    xs, _ = cbct.lsqr(cbct.Geometry(g), b.astype(np.float32), 30)
-    assert rel(x, xs) <= MIX_TOL
+        res = srv.wait(srv.submit(g, b, "lsqr", 30), timeout=300)
+    xs, rep = cbct.lsqr(cbct.Geometry(g), b.astype(np.float32), 30)
+    assert np.array_equal(np.asarray(res.report.resid), np.asarray(rep.resid))
+    assert np.array_equal(res.x, np.asarray(xs).reshape(res.x.shape))
