@@ -55,13 +55,13 @@ REF_STEP_ANGLES = 8             # --impl reference: about 7 s per step, so K ste
 # 360 from ncu (dram__bytes_read.sum + dram__bytes_write.sum, and
 # smsp__inst_executed.sum = warp instructions), keyed by the code of the
 # projector sources they were measured on (projector_hash(), comments
-# ignored) and the launch shape (rays per lane, transpose configuration);
-# the bench reports null once either differs.
+# ignored) and the launch shape (rays per lane, transpose configuration; each
+# kernel depends on its own); the bench reports null once either differs.
 NCU_COUNTERS = {
-    "forward": {"hash": "bf0c463e413182ae", "shape": [4, 3], "kernel": "forward_kernel<float, 0, 4, 1>",
-                "dram_bytes": 3018182400, "warp_inst": 19929252800},
-    "backward": {"hash": "bf0c463e413182ae", "shape": [4, 3], "kernel": "backward_kernel<float, 1, 2, 2, 1, 0>",
-                 "dram_bytes": 2791051008, "warp_inst": 31975031028},
+    "forward": {"hash": "08e3bee48d792b09", "shape": [4, 7], "kernel": "forward_kernel<float, 0, 4, 1, 1, 1>",
+                "dram_bytes": 1203765248, "warp_inst": 10792459808},
+    "backward": {"hash": "08e3bee48d792b09", "shape": [4, 7], "kernel": "patch_kernel<float, 1, 2, 0, 4, 1, 0>",
+                 "dram_bytes": 5919412480, "warp_inst": 10916571412},
 }
 
 # Instruction issue: one warp instruction per cycle per SM sub-partition.
@@ -257,15 +257,16 @@ def roofline_block(g, nnz, fwd_ms, bwd_ms, clocks, shape=None):
     instructions / issue peak): no L2 peak is measured on this machine (null),
     and the warp-instruction count comes from ncu (NCU_COUNTERS, null once the
     kernel source changed or when the run's launch shape `shape` = (rays per
-    lane, transpose configuration) is not the one the counters were taken
-    on)."""
+    lane, transpose configuration) is not the one the kernel's counters were
+    taken on)."""
     dominant = "forward" if fwd_ms >= bwd_ms else "backward"
     avg_ms = fwd_ms if dominant == "forward" else bwd_ms
     peak, peak_kind = measured_peak()
     achieved = nnz * BYTES_PER_UPDATE / (avg_ms * 1e-3) / 1e9
     c = NCU_COUNTERS.get(dominant)
+    own = 0 if dominant == "forward" else 1                  # the part of the launch shape the kernel depends on
     fresh = c is not None and c.get("hash") == projector_hash() and \
-        (shape is None or tuple(c.get("shape", ())) == tuple(shape))
+        (shape is None or c["shape"][own] == shape[own])
     warp_inst = c["warp_inst"] if fresh else None
     mhz = (clocks or {}).get("sm_mhz") or 2070.0
     issue_peak = SMS * SUBPARTITIONS * mhz * 1e6            # warp instructions per second

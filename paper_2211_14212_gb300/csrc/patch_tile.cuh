@@ -24,8 +24,8 @@
 //   is a small part of the sum, so nothing cancels.
 //
 // A^T y at 256^3 / 512^2 / 360 angles: 37.3 ms with backward_tile, 12.6 here;
-// 56 warp instructions per 32 voxels and angle, 63 in the first version
-// (169 in backward_tile), issue slots 76 % busy, 70 % of the sectors from L1.
+// 58 warp instructions per 32 voxels and angle, 63 in the first version
+// (169 in backward_tile), issue slots 72 % busy, 71 % of the sectors from L1.
 // Relative error against FP64 6.8e-7 -> 5.3e-7: fewer and shorter sums.
 // Measured and not kept: prefetching the next column's rows (2.87 against 2.80
 // ms per 90 angles) or the next angle's lines (3.48), four voxels per lane

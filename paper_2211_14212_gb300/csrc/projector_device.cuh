@@ -389,7 +389,7 @@ __device__ __forceinline__ RayZ make_rayz(const RayAxis &rz, float dz, int nz, b
 // A x at 256^3 / 512^2 / 360 angles: 24.2 -> 12.9 ms, 24 -> 12.6 warp
 // instructions per cell and 32 rays (two loads, one and a half packed FMA
 // pairs and an add for the sums, two for t and the plane, the rest address and
-// list), issue slots 62 % busy and L1 data wavefronts 54 %.
+// list), issue slots 67 % busy and L1 data wavefronts 54 %.
 template <typename T, bool COMP, int R, bool OFF32, int DIR, bool CLAMP>
 __device__ __forceinline__ void walk_cells(const DevGeom &g, const T *__restrict__ vol, CellList &cl, float amin,
                                            const RayZ (&z)[R], float4 *list, float (&acc)[R]) {
